@@ -2064,13 +2064,15 @@ int srbe_mlp_gradients(srbe_ctx *c, const float *D, const float *target, int64_t
     SRBE_REQUIRE(D && target && grad && n > 0, SRBE_EINVAL, "bad arguments");
     SRBE_REQUIRE(c->mlp.ready, SRBE_ESTATE, "no MLP parameters");
     upload_rows(c, D, target, n);
-    const double l = mlp_grad_step(c, c->mlp.data_D.p, c->mlp.data_T.p, nullptr, n, c->mlp.grad.p, false, 0.f, 0.f);
+    double *dl = c->mlp.loss.ensure(1), l = 0.0;
+    mlp_grad_step(c, c->mlp.data_D.p, c->mlp.data_T.p, nullptr, n, c->mlp.grad.p, false, 0.f, 0.f, dl);
     int64_t ntrain = 0;
     // the trainable part is everything before the input mean
     ntrain = mlp_param_count() - 2 * mlp_input_width() - 2;
     SRBE_CUDA(cudaMemcpyAsync(grad, c->mlp.grad.p, sizeof(float) * ntrain, cudaMemcpyDeviceToHost, c->stream));
+    SRBE_CUDA(cudaMemcpyAsync(&l, dl, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     SRBE_CUDA(cudaStreamSynchronize(c->stream));
-    if (loss) *loss = l;
+    if (loss) *loss = l / (double)n;
   });
 }
 
@@ -2108,6 +2110,10 @@ int srbe_mlp_train(srbe_ctx *c, const float *D, const float *target, int64_t n, 
     upload_rows(c, D, target, n);
     c->mlp.rows.ensure((size_t)n);
     std::vector<int32_t> perm(n);
+    // per minibatch the sum of squared errors, read back once per epoch (no wait between minibatches)
+    const int64_t nbatch = (n + batch - 1) / batch;
+    std::vector<double> err2(nbatch);
+    double *dl = c->mlp.loss.ensure((size_t)nbatch);
     double last = 0.0;
     uint64_t ctr = 0;
     for (int e = 0; e < epochs; ++e) {
@@ -2120,16 +2126,16 @@ int srbe_mlp_train(srbe_ctx *c, const float *D, const float *target, int64_t n, 
         std::swap(perm[i], perm[j]);
       }
       SRBE_CUDA(cudaMemcpyAsync(c->mlp.rows.p, perm.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, c->stream));
-      double tot = 0.0;
-      int64_t seen = 0;
-      for (int64_t b0 = 0; b0 < n; b0 += batch) {
-        const int64_t nb = std::min<int64_t>(batch, n - b0);
-        const double l = mlp_grad_step(c, c->mlp.data_D.p, c->mlp.data_T.p, c->mlp.rows.p + b0, nb, nullptr, true,
-                                       lr, weight_decay);
-        tot += l * nb;
-        seen += nb;
+      for (int64_t k = 0; k < nbatch; ++k) {
+        const int64_t b0 = k * batch, nb = std::min<int64_t>(batch, n - b0);
+        mlp_grad_step(c, c->mlp.data_D.p, c->mlp.data_T.p, c->mlp.rows.p + b0, nb, nullptr, true, lr, weight_decay,
+                      dl + k);
       }
-      last = tot / seen;
+      SRBE_CUDA(cudaMemcpyAsync(err2.data(), dl, sizeof(double) * nbatch, cudaMemcpyDeviceToHost, c->stream));
+      SRBE_CUDA(cudaStreamSynchronize(c->stream));
+      double tot = 0.0;
+      for (double v : err2) tot += v;
+      last = tot / (double)n;
     }
     if (final_loss) *final_loss = last;
   });

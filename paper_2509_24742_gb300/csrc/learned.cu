@@ -9,10 +9,9 @@
 //   64..79  Re, Im of exp(-i k_z Z_j) S1(k_z) for k_z = 2 pi m / L_z, m = 1..8 (the lowest k_z modes
 //           that the symmetry-preserving set I keeps, Eqs. 15 and 24)
 // Inputs and the target are standardised with the training set's mean and spread, which are part of
-// the parameter vector.  Training minimises the mean squared error with AdamW; the per-site
-// backward pass accumulates each block's gradient in shared memory (every thread owns its rows, so
-// the sum order is fixed) and a second kernel adds the block gradients in block order and applies
-// the AdamW update.
+// the parameter vector.  Training minimises the mean squared error with AdamW; the activations of a
+// minibatch come from one kernel, the weight gradients (sums over the rows in a fixed order) and the
+// AdamW update from a second.
 #include "srbe_internal.cuh"
 #include "tc.cuh"
 
@@ -27,10 +26,6 @@ constexpr int oW1 = 0, oB1 = oW1 + kH * kIn, oW2 = oB1 + kH, oB2 = oW2 + kH * kH
 constexpr int kNtrain = oXm;     // trainable entries come first
 
 __device__ __forceinline__ float silu(float z) { return z / (1.f + __expf(-z)); }
-__device__ __forceinline__ float silu_grad(float z) {
-  const float s = 1.f / (1.f + __expf(-z));
-  return s * (1.f + z * (1.f - s));
-}
 
 // S_low[m] = sum_i q_i exp(i 2 pi m z_i / L_z), m = 1..8, one block, fixed order
 __global__ void k_low_modes(int64_t n, const double *__restrict__ z, const double *__restrict__ q, double invLz,
@@ -267,78 +262,323 @@ k_mlp_forward_tc(int64_t n, const float *__restrict__ D, const float *__restrict
   if (warp == 0) tc::tmem_dealloc(tbase, 256);
 }
 
-// forward + backward of the standardised MSE loss over rows [blockIdx.x * chunk, ...); the block's
-// gradient (trainable entries) goes to gpart[blockIdx.x][kNtrain], its loss to lpart[blockIdx.x]
-__global__ void __launch_bounds__(kH)
-k_mlp_backward(int64_t n, int64_t chunk, const int32_t *__restrict__ rows, const float *__restrict__ D,
-               const float *__restrict__ T, const float *__restrict__ P, float inv_n, float *__restrict__ gpart,
-               double *__restrict__ lpart) {
-  extern __shared__ float g[];            // kNtrain floats
-  __shared__ float x[kIn], z1s[kH], h1[kH], dz2[kH], red[kH / 32];
-  const int h = threadIdx.x;
-  for (int i = h; i < kNtrain; i += kH) g[i] = 0.f;
-  double loss = 0.0;
-  __syncthreads();
-  const int64_t r0 = (int64_t)blockIdx.x * chunk, r1 = min(n, r0 + chunk);
-  for (int64_t rr = r0; rr < r1; ++rr) {
-    const int64_t row = rows ? rows[rr] : rr;
-    if (h < kIn) x[h] = (D[row * kIn + h] - P[oXm + h]) / P[oXs + h];
-    __syncthreads();
-    float z1 = P[oB1 + h];
-    for (int k = 0; k < kIn; ++k) z1 = fmaf(P[oW1 + h * kIn + k], x[k], z1);
-    z1s[h] = z1;
-    h1[h] = silu(z1);
-    __syncthreads();
-    float z2 = P[oB2 + h];
-    for (int k = 0; k < kH; ++k) z2 = fmaf(P[oW2 + h * kH + k], h1[k], z2);
-    const float a2 = silu(z2);
-    float v = P[oW3 + h] * a2;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((h & 31) == 0) red[h >> 5] = v;
-    __syncthreads();
-    const float o3 = red[0] + red[1] + red[2] + red[3] + P[oB3];
-    const float t = (T[row] - P[oYm]) / P[oYs];
-    const float err = o3 - t;
-    if (h == 0) loss += (double)err * err;
-    const float dout = 2.f * err * inv_n;
-    // layer 3
-    g[oW3 + h] += dout * a2;
-    if (h == 0) g[oB3] += dout;
-    const float d2 = dout * P[oW3 + h] * silu_grad(z2);
-    dz2[h] = d2;
-    // layer 2: thread h owns row h of W2
-    for (int k = 0; k < kH; ++k) g[oW2 + h * kH + k] += d2 * h1[k];
-    g[oB2 + h] += d2;
-    __syncthreads();
-    // layer 1: dh1[h] = sum_k W2[k][h] dz2[k]
-    float dh1 = 0.f;
-    for (int k = 0; k < kH; ++k) dh1 = fmaf(P[oW2 + k * kH + h], dz2[k], dh1);
-    const float d1 = dh1 * silu_grad(z1s[h]);
-    for (int k = 0; k < kIn; ++k) g[oW1 + h * kIn + k] += d1 * x[k];
-    g[oB1 + h] += d1;
-    __syncthreads();
-  }
-  for (int i = h; i < kNtrain; i += kH) gpart[(int64_t)blockIdx.x * kNtrain + i] = g[i];
-  if (h == 0) lpart[blockIdx.x] = loss;
+// Training pass (forward + backward of the standardised MSE loss), FP32 on the CUDA cores, two kernels:
+//
+// k_mlp_rows: a block stages W1 and W2 in shared memory once (odd row strides: both the row reads of the
+//   forward pass and the column reads of the backward pass are free of bank conflicts) and walks tiles
+//   of R rows; thread (h, half) owns hidden unit h and half of each dot product, the R rows of a tile are
+//   R independent FMA chains that share every weight read.  It writes the activations the weight
+//   gradients need: x, h1, dz1, dz2 and dout a2 per row.
+// k_mlp_wgrad: the weight gradients as products over the rows, dz2^T h1 and dz1^T x, one 16 x 16 tile of
+//   an output matrix per block, four row groups per block added in order, so that the small reduction
+//   (a minibatch) still fills the GPU; bias, W3 and loss sums in blocks of their own.  With one row
+//   split the same kernel applies AdamW, else a third kernel adds the splits in order.
+//
+// One block per row chunk with the gradient in shared memory and the weights read from global memory
+// (every thread its own row: uncoalesced, and 32-way bank conflicts on the gradient) took 440 us per
+// 512-row minibatch on GB300, host synchronisation included.
+constexpr int kTrThreads = 256;
+constexpr int kW1s = kIn + 1, kW2s = kH + 1;            // shared-memory row strides (odd)
+constexpr int64_t kTrSplit = 1024;                       // rows per split of the weight gradients
+constexpr int64_t kTrChunk = 65536;                      // rows whose activations are kept at once
+constexpr int kTrStage = 128;                            // rows staged per step of k_mlp_wgrad
+constexpr int kTile = 16;
+constexpr int kTilesW2 = (kH / kTile) * (kH / kTile), kTilesW1 = (kH / kTile) * (kIn / kTile);
+constexpr int kColBlocks = 3 * kH / 32;                  // b1, b2, W3: 32 columns per block
+constexpr int kWgradBlocks = kTilesW2 + kTilesW1 + kColBlocks + 1;
+static_assert(kH % 32 == 0 && kIn % kTile == 0 && kTrStage % 8 == 0, "MLP sizes must match the gradient tiles");
+
+struct TrainAct {                                        // per-row activations of one chunk, row-major
+  float *x, *h1, *dz1, *dz2, *a3;                        // [n][kIn], [n][kH] x 4 (a3 = dout SiLU(z2))
+  float2 *out;                                           // (dout, err)
+};
+
+// the training pass takes the correctly scaled exponential (the fast one is 2 ulp and more off): its
+// cost is hidden behind the dot products, and the gradients come out closer to their 64-bit values
+__device__ __forceinline__ float silu_train(float z) { return z / (1.f + expf(-z)); }
+__device__ __forceinline__ float silu_grad_train(float z) {
+  const float s = 1.f / (1.f + expf(-z));
+  return s * (1.f + z * (1.f - s));
 }
 
-// sums the block gradients in block order; optionally applies AdamW (step t >= 1)
-__global__ void k_mlp_reduce_adamw(int nblk, const float *__restrict__ gpart, float *__restrict__ grad,
-                                   float *__restrict__ P, float *__restrict__ m1, float *__restrict__ m2, int t,
-                                   float lr, float wd, int apply) {
+template <int R>
+__global__ void __launch_bounds__(kTrThreads)
+k_mlp_rows(int64_t n, const int32_t *__restrict__ rows, const float *__restrict__ D, const float *__restrict__ T,
+           const float *__restrict__ P, float inv_n, TrainAct act) {
+  extern __shared__ float tsm[];
+  float *w1 = tsm, *w2 = w1 + kH * kW1s;
+  float *xs = w2 + kH * kW2s;                            // [kIn][R]
+  float *hs = xs + kIn * R, *ds = hs + kH * R;           // [kH][R] each: h1, then dz2
+  float *ps = ds + kH * R;                               // [kH][R]: the upper half's partial sums
+  __shared__ float wsum[4][R];
+  __shared__ float serr[R];
+  const int t = threadIdx.x, h = t & (kH - 1), half = t >> 7, lane = t & 31;
+  for (int i = t; i < kH * kIn; i += kTrThreads) w1[(i / kIn) * kW1s + i % kIn] = P[oW1 + i];
+  for (int i = t; i < kH * kH; i += kTrThreads) w2[(i / kH) * kW2s + i % kH] = P[oW2 + i];
+  const float b1 = P[oB1 + h], b2 = P[oB2 + h], w3 = P[oW3 + h], b3 = P[oB3], ym = P[oYm], ys = P[oYs];
+  const int64_t ntile = (n + R - 1) / R;
+  for (int64_t tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
+    const int64_t r0 = tile * R;
+    __syncthreads();                                     // weights staged / the last tile's buffers free
+    for (int i = t; i < kIn * R; i += kTrThreads) {
+      const int r = i / kIn, k = i - r * kIn;
+      float v = 0.f;
+      if (r0 + r < n) {
+        const int64_t row = rows ? rows[r0 + r] : r0 + r;
+        v = (D[row * kIn + k] - P[oXm + k]) / P[oXs + k];
+        act.x[(r0 + r) * kIn + k] = v;
+      }
+      xs[k * R + r] = v;
+    }
+    __syncthreads();
+    float z[R], z1[R], z2[R];
+    // layer 1
+#pragma unroll
+    for (int r = 0; r < R; ++r) z[r] = 0.f;
+    {
+      const int k0 = half * (kIn / 2);
+#pragma unroll 8
+      for (int k = 0; k < kIn / 2; ++k) {
+        const float w = w1[h * kW1s + k0 + k];
+#pragma unroll
+        for (int r = 0; r < R; ++r) z[r] = fmaf(w, xs[(k0 + k) * R + r], z[r]);
+      }
+    }
+    if (half) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) ps[h * R + r] = z[r];
+    }
+    __syncthreads();
+    if (!half) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        z1[r] = b1 + (z[r] + ps[h * R + r]);
+        hs[h * R + r] = silu_train(z1[r]);
+      }
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+        if (r0 + r < n) act.h1[(r0 + r) * kH + h] = hs[h * R + r];
+    }
+    __syncthreads();
+    // layer 2
+#pragma unroll
+    for (int r = 0; r < R; ++r) z[r] = 0.f;
+    {
+      const int k0 = half * (kH / 2);
+#pragma unroll 8
+      for (int k = 0; k < kH / 2; ++k) {
+        const float w = w2[h * kW2s + k0 + k];
+#pragma unroll
+        for (int r = 0; r < R; ++r) z[r] = fmaf(w, hs[(k0 + k) * R + r], z[r]);
+      }
+    }
+    if (half) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) ps[h * R + r] = z[r];
+    }
+    __syncthreads();
+    if (!half) {
+      // output: the four warps of this half add W3 . SiLU(z2) over the hidden units
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        z2[r] = b2 + (z[r] + ps[h * R + r]);
+        float v = w3 * silu_train(z2[r]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) wsum[h >> 5][r] = v;
+      }
+    }
+    __syncthreads();
+    if (t < R) {
+      const float o3 = wsum[0][t] + wsum[1][t] + wsum[2][t] + wsum[3][t] + b3;
+      float err = 0.f;
+      if (r0 + t < n) {
+        const int64_t row = rows ? rows[r0 + t] : r0 + t;
+        err = o3 - (T[row] - ym) / ys;
+        act.out[r0 + t] = make_float2(2.f * err * inv_n, err);
+      }
+      serr[t] = err;
+    }
+    __syncthreads();
+    if (!half) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const float dout = 2.f * serr[r] * inv_n;
+        const float d2 = dout * w3 * silu_grad_train(z2[r]);
+        ds[h * R + r] = d2;
+        if (r0 + r < n) {
+          act.dz2[(r0 + r) * kH + h] = d2;
+          act.a3[(r0 + r) * kH + h] = dout * silu_train(z2[r]);
+        }
+      }
+    }
+    __syncthreads();
+    // dh1[h] = sum_k W2[k][h] dz2[k]
+#pragma unroll
+    for (int r = 0; r < R; ++r) z[r] = 0.f;
+    {
+      const int k0 = half * (kH / 2);
+#pragma unroll 8
+      for (int k = 0; k < kH / 2; ++k) {
+        const float w = w2[(k0 + k) * kW2s + h];
+#pragma unroll
+        for (int r = 0; r < R; ++r) z[r] = fmaf(w, ds[(k0 + k) * R + r], z[r]);
+      }
+    }
+    if (half) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) ps[h * R + r] = z[r];
+    }
+    __syncthreads();
+    if (!half) {
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+        if (r0 + r < n) act.dz1[(r0 + r) * kH + h] = (z[r] + ps[h * R + r]) * silu_grad_train(z1[r]);
+    }
+  }
+}
+
+struct AdamW {
+  float *P, *m1, *m2;
+  int t;
+  float lr, wd;
+};
+// one AdamW update of parameter i with gradient s
+__device__ __forceinline__ void adamw_update(const AdamW &a, int i, float s) {
+  const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
+  const float m = b1 * a.m1[i] + (1.f - b1) * s, v = b2 * a.m2[i] + (1.f - b2) * s * s;
+  a.m1[i] = m;
+  a.m2[i] = v;
+  const float mh = m / (1.f - powf(b1, (float)a.t)), vh = v / (1.f - powf(b2, (float)a.t));
+  a.P[i] -= a.lr * (mh / (sqrtf(vh) + eps) + a.wd * a.P[i]);
+}
+
+// weight gradients over the rows of split blockIdx.y of the chunk; fused: the only split, so each
+// gradient goes to grad (if given) and into AdamW (if apply), else to gpart[slot0 + split]
+__global__ void __launch_bounds__(kTrThreads)
+k_mlp_wgrad(int64_t n, TrainAct act, float *__restrict__ gpart, double *__restrict__ lpart, int64_t slot0, int fused,
+            float *__restrict__ grad, int apply, AdamW opt) {
+  __shared__ __align__(16) float sa[kTrStage][kTile], sb[kTrStage][kTile];
+  __shared__ float red[4][kTile * kTile];
+  const int t = threadIdx.x, blk = blockIdx.x;
+  const int64_t r0 = (int64_t)blockIdx.y * kTrSplit, r1 = min(n, r0 + kTrSplit);
+  const int64_t slot = slot0 + blockIdx.y;
+  auto put = [&](int i, float s) {
+    if (!fused) {
+      gpart[slot * kNtrain + i] = s;
+      return;
+    }
+    if (grad) grad[i] = s;
+    if (apply) adamw_update(opt, i, s);
+  };
+  if (blk < kTilesW2 + kTilesW1) {
+    // 16 x 16 outputs: g[h0 + i][k0 + j] = sum_r A[r][h0 + i] B[r][k0 + j]
+    const bool second = blk < kTilesW2;
+    const int tl = second ? blk : blk - kTilesW2, across = second ? kH / kTile : kIn / kTile;
+    const int h0 = (tl / across) * kTile, k0 = (tl % across) * kTile;
+    const float *A = second ? act.dz2 : act.dz1, *B = second ? act.h1 : act.x;
+    const int ldb = second ? kH : kIn;
+    const int grp = t >> 6, i2 = 2 * ((t & 63) >> 3), j2 = 2 * (t & 7);
+    float g00 = 0.f, g01 = 0.f, g10 = 0.f, g11 = 0.f;
+    // a stage's loads: each thread two rows' 16-byte pieces of A and of B, fetched one stage ahead
+    const int lr = t >> 2, lc = 4 * (t & 3);
+    float4 pa[2], pb[2];
+    auto fetch = [&](int64_t base) {
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int64_t r = base + lr + 64 * u;
+        const bool ok = r < r1;
+        pa[u] = ok ? __ldcg(reinterpret_cast<const float4 *>(A + r * kH + h0 + lc)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        pb[u] = ok ? __ldcg(reinterpret_cast<const float4 *>(B + r * ldb + k0 + lc)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    };
+    fetch(r0);
+    for (int64_t base = r0; base < r1; base += kTrStage) {
+      __syncthreads();
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        *reinterpret_cast<float4 *>(&sa[lr + 64 * u][lc]) = pa[u];
+        *reinterpret_cast<float4 *>(&sb[lr + 64 * u][lc]) = pb[u];
+      }
+      __syncthreads();
+      if (base + kTrStage < r1) fetch(base + kTrStage);
+#pragma unroll 8
+      for (int r = grp; r < kTrStage; r += 4) {          // rows beyond r1 are zero
+        const float2 a = *reinterpret_cast<const float2 *>(&sa[r][i2]);
+        const float2 b = *reinterpret_cast<const float2 *>(&sb[r][j2]);
+        g00 = fmaf(a.x, b.x, g00);
+        g01 = fmaf(a.x, b.y, g01);
+        g10 = fmaf(a.y, b.x, g10);
+        g11 = fmaf(a.y, b.y, g11);
+      }
+    }
+    red[grp][i2 * kTile + j2] = g00;
+    red[grp][i2 * kTile + j2 + 1] = g01;
+    red[grp][(i2 + 1) * kTile + j2] = g10;
+    red[grp][(i2 + 1) * kTile + j2 + 1] = g11;
+    __syncthreads();
+    const float s = ((red[0][t] + red[1][t]) + red[2][t]) + red[3][t];
+    put((second ? oW2 : oW1) + (h0 + t / kTile) * (second ? kH : kIn) + k0 + t % kTile, s);
+  } else if (blk < kTilesW2 + kTilesW1 + kColBlocks) {
+    // column sums: 32 columns x 8 row groups, added in group order
+    const int cb = blk - kTilesW2 - kTilesW1, what = cb / (kH / 32), c0 = (cb % (kH / 32)) * 32;
+    const float *A = what == 0 ? act.dz1 : (what == 1 ? act.dz2 : act.a3);
+    const int col = t & 31, grp = t >> 5;
+    float s = 0.f;
+#pragma unroll 16
+    for (int64_t r = r0 + grp; r < r1; r += 8) s += __ldcg(A + r * kH + c0 + col);
+    float *rs = &red[0][0];
+    rs[t] = s;
+    __syncthreads();
+    if (t < 32) {
+      float v = rs[t];
+#pragma unroll
+      for (int g = 1; g < 8; ++g) v += rs[32 * g + t];
+      put((what == 0 ? oB1 : (what == 1 ? oB2 : oW3)) + c0 + t, v);
+    }
+  } else {
+    // b3 and the loss
+    __shared__ double dred[kTrThreads];
+    float s = 0.f;
+    double l = 0.0;
+    for (int64_t r = r0 + t; r < r1; r += kTrThreads) {
+      const float2 o = __ldcg(act.out + r);
+      s += o.x;
+      l += (double)o.y * (double)o.y;
+    }
+    float *rs = &red[0][0];
+    rs[t] = s;
+    dred[t] = l;
+    __syncthreads();
+    for (int o = kTrThreads / 2; o > 0; o >>= 1) {
+      if (t < o) {
+        rs[t] += rs[t + o];
+        dred[t] += dred[t + o];
+      }
+      __syncthreads();
+    }
+    if (t == 0) {
+      put(oB3, rs[0]);
+      lpart[fused ? 0 : slot] = dred[0];
+    }
+  }
+}
+
+// adds the splits' gradients (and squared errors) in order; optionally applies AdamW
+__global__ void k_mlp_reduce(int64_t nslot, const float *__restrict__ gpart, const double *__restrict__ lpart,
+                             double *__restrict__ loss, float *__restrict__ grad, int apply, AdamW opt) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0) {
+    double l = 0.0;
+    for (int64_t b = 0; b < nslot; ++b) l += lpart[b];
+    *loss = l;
+  }
   if (i >= kNtrain) return;
   float s = 0.f;
-  for (int b = 0; b < nblk; ++b) s += gpart[(int64_t)b * kNtrain + i];
+#pragma unroll 8
+  for (int64_t b = 0; b < nslot; ++b) s += gpart[b * kNtrain + i];
   if (grad) grad[i] = s;
-  if (!apply) return;
-  const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-  const float a = b1 * m1[i] + (1.f - b1) * s, v = b2 * m2[i] + (1.f - b2) * s * s;
-  m1[i] = a;
-  m2[i] = v;
-  const float ah = a / (1.f - powf(b1, (float)t)), vh = v / (1.f - powf(b2, (float)t));
-  P[i] -= lr * (ah / (sqrtf(vh) + eps) + wd * P[i]);
+  if (apply) adamw_update(opt, i, s);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -374,33 +614,61 @@ void mlp_forward(srbe_ctx *c, const float *D_dev, int64_t n, float *out_dev, dou
   SRBE_CUDA(cudaGetLastError());
 }
 
-// gradient (and optionally one AdamW step) over rows (all n rows when rows_dev is null)
-double mlp_grad_step(srbe_ctx *c, const float *D_dev, const float *T_dev, const int32_t *rows_dev, int64_t n,
-                     float *grad_dev, bool apply, float lr, float wd) {
+// gradient (and optionally one AdamW step) over rows (all n rows when rows_dev is null); the sum of the
+// squared standardised errors goes to *loss_dev.  Queued on the context's stream.
+void mlp_grad_step(srbe_ctx *c, const float *D_dev, const float *T_dev, const int32_t *rows_dev, int64_t n,
+                   float *grad_dev, bool apply, float lr, float wd, double *loss_dev) {
   auto &m = c->mlp;
-  const int nblk = (int)std::max<int64_t>(1, std::min<int64_t>(152, (n + 15) / 16));
-  const int64_t chunk = (n + nblk - 1) / nblk;
-  m.gpart.ensure((size_t)nblk * kNtrain);
-  m.lpart.ensure((size_t)nblk);
-  const size_t smem = sizeof(float) * kNtrain;
-  static bool attr = false;
-  if (!attr) {
-    SRBE_CUDA(cudaFuncSetAttribute(k_mlp_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    attr = true;
+  static int nsm = 0;
+  constexpr size_t kRowsSmem4 = sizeof(float) * (kH * (kW1s + kW2s) + 4 * (kIn + 3 * kH));
+  constexpr size_t kRowsSmem8 = sizeof(float) * (kH * (kW1s + kW2s) + 8 * (kIn + 3 * kH));
+  if (!nsm) {
+    int dev = 0, v = 0;
+    SRBE_CUDA(cudaGetDevice(&dev));
+    SRBE_CUDA(cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev));
+    SRBE_CUDA(cudaFuncSetAttribute(k_mlp_rows<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowsSmem4));
+    SRBE_CUDA(cudaFuncSetAttribute(k_mlp_rows<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowsSmem8));
+    nsm = v;
   }
-  k_mlp_backward<<<nblk, kH, smem, c->stream>>>(n, chunk, rows_dev, D_dev, T_dev, m.P.p, 1.0f / (float)n, m.gpart.p,
-                                                m.lpart.p);
+  const int64_t nslot = (n + kTrSplit - 1) / kTrSplit, most = std::min(n, kTrChunk);
+  const bool fused = nslot == 1;
+  const int64_t rows_max = (most + 3) & ~(int64_t)3;     // keeps every array on a 16-byte boundary
+  float *buf = m.act.ensure((size_t)rows_max * (kIn + 4 * kH + 2));
+  TrainAct act;
+  act.out = reinterpret_cast<float2 *>(buf);
+  act.x = buf + 2 * rows_max;
+  act.h1 = act.x + kIn * rows_max;
+  act.dz1 = act.h1 + kH * rows_max;
+  act.dz2 = act.dz1 + kH * rows_max;
+  act.a3 = act.dz2 + kH * rows_max;
+  if (!fused) {
+    m.gpart.ensure((size_t)nslot * kNtrain);
+    m.lpart.ensure((size_t)nslot);
+  }
   if (apply) m.t++;
-  k_mlp_reduce_adamw<<<blocks_for(kNtrain, 256), 256, 0, c->stream>>>(nblk, m.gpart.p, grad_dev, m.P.p, m.m1.p, m.m2.p,
-                                                                      m.t, lr, wd, apply ? 1 : 0);
-  c->launches += 2;
+  const AdamW opt{m.P.p, m.m1.p, m.m2.p, m.t, lr, wd};
+  for (int64_t b0 = 0; b0 < n; b0 += kTrChunk) {
+    const int64_t nb = std::min(kTrChunk, n - b0);
+    const int32_t *rows = rows_dev ? rows_dev + b0 : nullptr;
+    const float *D = rows_dev ? D_dev : D_dev + b0 * kIn, *T = rows_dev ? T_dev : T_dev + b0;
+    // 4 rows per tile while one wave of blocks covers them (a 512-row minibatch: 128 blocks), then 8
+    if (nb <= 4 * (int64_t)nsm)
+      k_mlp_rows<4><<<(unsigned)((nb + 3) / 4), kTrThreads, kRowsSmem4, c->stream>>>(nb, rows, D, T, m.P.p,
+                                                                                    1.0f / (float)n, act);
+    else
+      k_mlp_rows<8><<<(unsigned)std::min<int64_t>((nb + 7) / 8, nsm), kTrThreads, kRowsSmem8, c->stream>>>(
+          nb, rows, D, T, m.P.p, 1.0f / (float)n, act);
+    const unsigned splits = (unsigned)((nb + kTrSplit - 1) / kTrSplit);
+    k_mlp_wgrad<<<dim3(kWgradBlocks, splits), kTrThreads, 0, c->stream>>>(
+        nb, act, m.gpart.p, fused ? loss_dev : m.lpart.p, b0 / kTrSplit, fused ? 1 : 0, grad_dev, apply ? 1 : 0, opt);
+    c->launches += 2;
+  }
+  if (!fused) {
+    k_mlp_reduce<<<blocks_for(kNtrain, 128), 128, 0, c->stream>>>(nslot, m.gpart.p, m.lpart.p, loss_dev, grad_dev,
+                                                                  apply ? 1 : 0, opt);
+    c->launches++;
+  }
   SRBE_CUDA(cudaGetLastError());
-  std::vector<double> lp(nblk);
-  SRBE_CUDA(cudaMemcpyAsync(lp.data(), m.lpart.p, sizeof(double) * nblk, cudaMemcpyDeviceToHost, c->stream));
-  SRBE_CUDA(cudaStreamSynchronize(c->stream));
-  double l = 0.0;
-  for (double v : lp) l += v;
-  return l / (double)n;
 }
 
 }  // namespace srbe

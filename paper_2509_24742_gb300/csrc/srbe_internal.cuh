@@ -123,7 +123,8 @@ struct MlpState {
   bool ready = false;
   int t = 0;
   DevBuf<float> P, m1, m2, gpart, grad, D, data_D, data_T;
-  DevBuf<double> lpart;
+  DevBuf<float> act;                 // activations of a training pass, row-major
+  DevBuf<double> lpart, loss;        // squared errors: per split, per minibatch of an epoch
   DevBuf<double2> Slow;
   DevBuf<int32_t> rows;
 };
@@ -412,8 +413,8 @@ int mlp_param_count();
 int mlp_input_width();
 void mlp_descriptors(srbe_ctx *c, float *D_dev);
 void mlp_forward(srbe_ctx *c, const float *D_dev, int64_t n, float *out_dev, double *out_y_dev);
-double mlp_grad_step(srbe_ctx *c, const float *D_dev, const float *T_dev, const int32_t *rows_dev, int64_t n,
-                     float *grad_dev, bool apply, float lr, float wd);
+void mlp_grad_step(srbe_ctx *c, const float *D_dev, const float *T_dev, const int32_t *rows_dev, int64_t n,
+                   float *grad_dev, bool apply, float lr, float wd, double *loss_dev);
 void ion_forces(srbe_ctx *c, bool energies);
 bool ion_forces_split(const srbe_ctx *c, bool energies);
 void ion_forces_ii(srbe_ctx *c);
