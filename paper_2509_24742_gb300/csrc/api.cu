@@ -552,6 +552,7 @@ void reserve(srbe_ctx *c) {
   nb.xb.ensure(nn);
   nb.yb.ensure(nn);
   nb.pfb.ensure(nn);
+  if (c->have_md) nb.pm.ensure(nn);
   nb.cell_s.ensure(nn);
   nb.flag.ensure(3);
   if (c->lat.nl > 0) c->lat.E.ensure((size_t)K * c->lat.nl);

@@ -100,6 +100,7 @@ struct NbrLists {
   int cap = 0;
   DevBuf<double> xb, yb;             // sorted x, y at the last build (unwrapping reference)
   DevBuf<float4> pfb;                // sorted FP32 positions at the last build
+  DevBuf<float4> pm;                 // the same with the molecule id's bits (MD): the list build's candidates
   DevBuf<int32_t> cell_s;            // cell of each sorted ion at the last build
   DevBuf<int> flag;                  // [0] rebuild needed, [1] forced by the host, [2] list-task counter
   double skin = 0.1;
