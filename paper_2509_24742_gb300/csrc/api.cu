@@ -253,12 +253,16 @@ __global__ void k_deinterleave(int64_t n, const double *__restrict__ r, double L
 }
 
 __global__ void k_site_turns(int64_t n, const double *__restrict__ x, const double *__restrict__ y,
-                             const double *__restrict__ z, double3 invL, uint64_t *__restrict__ u) {
+                             const double *__restrict__ z, double3 invL, uint64_t *__restrict__ u, double invW,
+                             uint64_t *__restrict__ uw) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   u[i] = to_turns64(x[i], invL.x);
   u[n + i] = to_turns64(y[i], invL.y);
   u[2 * n + i] = to_turns64(z[i], invL.z);
+  uw[i] = to_turns64_exact(x[i], invW);
+  uw[n + i] = to_turns64_exact(y[i], invW);
+  uw[2 * n + i] = to_turns64_exact(z[i], invW);
 }
 
 // FP32 copies of the fixed site positions (the mixed form's b), site order
@@ -534,6 +538,10 @@ void reserve(srbe_ctx *c) {
   cl.ms.ensure(nn);
   cl.pf.ensure(nn);
   cl.us.ensure(3 * nn);
+  if (c->precision == SRBE_FP64) {
+    cl.uw.ensure(3 * nn);
+    pair_tables(c);
+  }
   NbrLists &nb = c->nbr;
   if (nb.cap == 0) {
     // twice the expected neighbour count at rc + skin for the mean ion density between the walls
@@ -1327,7 +1335,7 @@ int srbe_set_electrode(srbe_ctx *c, int64_t n_ele, const double *R, const int8_t
     k_site_turns<<<blocks_for(n_ele, 256), 256, 0, c->stream>>>(n_ele, c->ex.p, c->ey.p, c->ez.p,
                                                                make_double3(1.0 / c->L[0], 1.0 / c->L[1],
                                                                             1.0 / c->L[2]),
-                                                               c->eu.p);
+                                                               c->eu.p, 1.0 / pair_period(c), c->euw.ensure(3 * (size_t)n_ele));
     k_site_f4<<<blocks_for(n_ele, 256), 256, 0, c->stream>>>(n_ele, c->ex.p, c->ey.p, c->ez.p,
                                                             c->epf.ensure((size_t)n_ele));
     SRBE_CUDA(cudaGetLastError());
@@ -1474,6 +1482,15 @@ int srbe_set_md(srbe_ctx *c, const double *mass, const double *v, int ntype, con
     c->itype.ensure(nn);
     c->mol.ensure(nn);
     c->lj.ensure(lj.size());
+    // the FP64 form's pair sums: 24 eps (2 sr^12 - sr^6) / r^2 = (A u^3 - B) u^4 with u = (R1 / r)^2, R1 = W / 8
+    std::vector<double> ljp(lj.size());
+    const double R2 = std::pow(0.125 * pair_period(c), 2);
+    for (int a = 0; a < ntype * ntype; ++a) {
+      const double s2 = lj[2 * a] / R2, s6 = s2 * s2 * s2;
+      ljp[2 * a] = 48.0 * lj_eps[a] * (s6 * s6) / R2;
+      ljp[2 * a + 1] = 24.0 * lj_eps[a] * s6 / R2;
+    }
+    c->ljp.ensure(ljp.size());
     c->bond_start.ensure(n + 1);
     c->bond_j.ensure(std::max<int64_t>(2 * nb, 1));
     c->bond_r0.ensure(std::max<int64_t>(2 * nb, 1));
@@ -1493,6 +1510,7 @@ int srbe_set_md(srbe_ctx *c, const double *mass, const double *v, int ntype, con
       SRBE_CUDA(cudaMemcpy(c->mol.p, mol, sizeof(int32_t) * n, cudaMemcpyHostToDevice));
     }
     SRBE_CUDA(cudaMemcpy(c->lj.p, lj.data(), sizeof(double) * lj.size(), cudaMemcpyHostToDevice));
+    SRBE_CUDA(cudaMemcpy(c->ljp.p, ljp.data(), sizeof(double) * ljp.size(), cudaMemcpyHostToDevice));
     std::vector<float> lj32(lj.begin(), lj.end());
     c->lj32.ensure(lj32.size() / 2);
     SRBE_CUDA(cudaMemcpy(c->lj32.p, lj32.data(), sizeof(float) * lj32.size(), cudaMemcpyHostToDevice));

@@ -138,8 +138,10 @@ struct Cells {
   DevBuf<int32_t> ts, ms;                     // type, molecule in sorted order
   DevBuf<float4> pf;                          // FP32 (x, y, z, w) in sorted order for the pre-check
   DevBuf<uint64_t> us;                        // fixed-point phase coordinates [3][n] in sorted order
+  DevBuf<uint64_t> uw;                        // pair coordinates [3][n], fractions of the period W (FP64 form)
 };
 
+struct PairCoef;  // one interval of a radial table (pairfix.cuh)
 struct HostExt;   // host-only per-context state (sampler, staging), defined in api.cu
 
 }  // namespace srbe
@@ -204,6 +206,7 @@ struct srbe_ctx {
   int64_t ne = 0;
   srbe::DevBuf<double> ex, ey, ez, ed;         // positions and d (-1/2 | +1/2)
   srbe::DevBuf<uint64_t> eu;                   // fixed-point phase coordinates [3][ne], site order
+  srbe::DevBuf<uint64_t> euw;                  // pair coordinates [3][ne], site order (FP64 form)
   srbe::DevBuf<float4> epf;                    // FP32 site positions (x, y, z, 0), site order
   srbe::DevBuf<uint64_t> iu;                   // ion phase coordinates [3][ni] written by the drift of a step
   srbe::DevBuf<double> Bmat;                   // projected inverse J A^-1, ne x ne row-major
@@ -234,6 +237,9 @@ struct srbe_ctx {
   srbe::DevBuf<double> bond_r0;
   int ntype = 0;
   srbe::DevBuf<double> lj;                     // [ntype*ntype] (sigma^2, 4 eps) pairs as double2
+  srbe::DevBuf<double> ljp;                    // [ntype*ntype] (A, B) of the FP64 form's pair sums
+  srbe::DevBuf<srbe::PairCoef> ptab;           // the FP64 form's radial tables: ion-ion, ion-electrode, phi_ie
+  bool ptab_ready = false;
   double kb = 0, dt = 0;
   srbe::Cells icells;
 
@@ -349,6 +355,13 @@ __device__ __forceinline__ uint64_t to_turns64(double x, double invL) {
   return (uint64_t)__double2ull_rz(t * 18446744073709551616.0);
 }
 
+// frac(x / W) 2^64 for a power-of-two W given as its (exact) inverse: exact for either sign up to the last
+// unit (the sign is taken off first, since 1 - small would round)
+__device__ __forceinline__ uint64_t to_turns64_exact(double x, double invW) {
+  const uint64_t u = to_turns64(fabs(x), invW);
+  return x < 0.0 ? 0ull - u : u;
+}
+
 __device__ __forceinline__ uint64_t phase64(int4 m, uint64_t ux, uint64_t uy, uint64_t uz) {
   return (uint64_t)(int64_t)m.x * ux + (uint64_t)(int64_t)m.y * uy + (uint64_t)(int64_t)m.z * uz;
 }
@@ -395,6 +408,9 @@ __device__ __forceinline__ void sincos_turns32(uint32_t th, float &c, float &s) 
 // kernels' host launchers (defined in the .cu files)
 // ------------------------------------------------------------------------------------------------
 void upload_table(srbe_ctx *c);
+// the FP64 form's pair sums: the period W of its fixed-point coordinates and its radial tables
+double pair_period(const srbe_ctx *c);
+void pair_tables(srbe_ctx *c);
 void build_cells(srbe_ctx *c, Cells &cl, int64_t n, const double *x, const double *y, const double *z,
                  const double *w, const int32_t *typ, const int32_t *mol, bool is_ion);
 void choose_grid(const srbe_ctx *c, CellGrid &g, double zlo, double zhi);
