@@ -540,6 +540,7 @@ void reserve(srbe_ctx *c) {
   cl.us.ensure(3 * nn);
   if (c->precision == SRBE_FP64) {
     cl.uw.ensure(3 * nn);
+    c->kv.ensure((size_t)3 * K);
     pair_tables(c);
   }
   NbrLists &nb = c->nbr;

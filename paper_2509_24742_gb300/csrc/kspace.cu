@@ -53,6 +53,8 @@ struct SfFinish {
   double2 *coef;
   float2 *coef32;
   int swap;
+  double *kv;               // not null: the modes as doubles, for the force gather
+  const int4 *modes;
 };
 
 __device__ __forceinline__ void sf_finish(const SfFinish &f, int k, int lane) {
@@ -84,6 +86,7 @@ __device__ __forceinline__ void sf_finish(const SfFinish &f, int k, int lane) {
         const double2 v = f.swap ? make_double2(c * im, c * re) : make_double2(c * re, c * im);
         f.coef[k] = v;
         f.coef32[k] = make_float2((float)v.x, (float)v.y);
+        if (f.kv) store_mode(f.kv, f.K, k, f.modes[k]);
       }
     } else {
       f.scal[f.mslot] = re;
@@ -137,7 +140,7 @@ k_sfac_partial(int64_t n, const double *__restrict__ x, const double *__restrict
     if (!F32) {
       for (int j = warp; j < cnt; j += 4) {
         double c, s;
-        sincos_turns(phase64(m, su[0][j], su[1][j], su[2][j]), tab, c, s);
+        sincos_turns_fix(phase64(m, su[0][j], su[1][j], su[2][j]), tab, c, s);
         are = fma(sw[j], c, are);
         aim = fma(sw[j], s, aim);
       }
@@ -282,6 +285,7 @@ k_sfac_partial(int64_t n, const double *__restrict__ x, const double *__restrict
       const double2 v = fin.swap ? make_double2(c * im, c * re) : make_double2(c * re, c * im);
       fin.coef[kidx] = v;
       fin.coef32[kidx] = make_float2((float)v.x, (float)v.y);
+      if (fin.kv) store_mode(fin.kv, K, kidx, m);
     }
   }
   if (blockIdx.y == 0 && warp == 1) sf_finish(fin, K, lane);     // the dipole partials
@@ -335,7 +339,8 @@ void structure_factor(srbe_ctx *c, int64_t n, const double *x, const double *y, 
                SRBE_ESTATE, "scratch buffers not reserved for this size");
   const double3 invL = make_double3(1.0 / c->L[0], 1.0 / c->L[1], 1.0 / c->L[2]);
   SfFinish f{K, (int)nchunk, c->partial.p, c->mpart.p, S, S_add, c->scal.p, mslot, c->dc.p,
-             coef_mode >= 0 ? c->coef.p : nullptr, c->coef32.p, coef_mode > 0 ? 1 : 0};
+             coef_mode >= 0 ? c->coef.p : nullptr, c->coef32.p, coef_mode > 0 ? 1 : 0,
+             coef_mode > 0 && c->precision == SRBE_FP64 ? c->kv.p : nullptr, c->dm.p};
   if (nchunk > 0) {
     SRBE_REQUIRE(c->sfdone.cap >= (size_t)ktiles, SRBE_ESTATE, "tile counters not reserved for this size");
     dim3 grid((unsigned)nchunk, (unsigned)ktiles);

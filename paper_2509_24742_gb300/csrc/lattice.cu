@@ -145,7 +145,7 @@ __global__ void k_lat_modes(LatDev L, int K, const int4 *__restrict__ modes, con
                             const double2 *__restrict__ E, const double *__restrict__ Zl,
                             const double2 *__restrict__ S1, const double *__restrict__ cw, double2 *__restrict__ S,
                             double2 *__restrict__ coef, float2 *__restrict__ coef32, double *__restrict__ scal,
-                            int mslot) {
+                            int mslot, double *__restrict__ kv) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k > K) return;
   if (k == K) {
@@ -170,6 +170,7 @@ __global__ void k_lat_modes(LatDev L, int K, const int4 *__restrict__ modes, con
   const double2 v = make_double2(c * im, c * re);
   coef[k] = v;
   coef32[k] = make_float2((float)v.x, (float)v.y);
+  if (kv) store_mode(kv, K, k, m);
 }
 
 // one warp per bin (a, b): W_l[b][a] = sum over the modes of the bin of (c S1)(k) conj(E[k][l]);
@@ -351,7 +352,8 @@ void lattice_s2(srbe_ctx *c, double2 *S, const double2 *S1, int mslot) {
   launch_line<kFwdY>(c, L, c->lat.T.p, c->lat.Qh.p);
   k_lat_modes<<<blocks_for(c->K + 1, 64), 64, 0, c->stream>>>(L, c->K, c->dm.p, c->lat.Qh.p, c->lat.E.p, c->lat.Zl.p,
                                                                 S1, c->dc.p, S, c->coef.p, c->coef32.p, c->scal.p,
-                                                                mslot);
+                                                                mslot,
+                                                                c->precision == SRBE_FP64 ? c->kv.p : nullptr);
   c->launches += 1;
   c->mode_evals += (int64_t)c->K * L.nl;
   SRBE_CUDA(cudaGetLastError());

@@ -61,7 +61,7 @@ k_na_partial(int64_t n, const double *__restrict__ r, const double *__restrict__
     const int cnt = (int)min((int64_t)kNaThreads, i1 - base);
     for (int j = warp; j < cnt; j += 4) {
       double c, s;
-      sincos_turns(phase64(m, su[0][j], su[1][j], su[2][j]), tab, c, s);
+      sincos_turns_fix(phase64(m, su[0][j], su[1][j], su[2][j]), tab, c, s);
       are = fma(sw[j], c, are);
       aim = fma(sw[j], s, aim);
     }

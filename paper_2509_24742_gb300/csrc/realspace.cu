@@ -562,8 +562,9 @@ __device__ __forceinline__ void pair_ion_ion_fix(const PairSite &S, const CellsD
     return;
   }
   const PairArg p = pair_arg(Sv);
-  double fs = S.qi * ions.ws[e.x] * pair_poly(fx.ii[p.idx], p);
-  if (md.ntype && ions.ms[e.x] != S.mi) fs += pair_lj(md.ljp[S.ti * md.ntype + ions.ts[e.x]], p, Sv);
+  double lj = 0.0;
+  if (md.ntype && ions.ms[e.x] != S.mi) lj = pair_lj(md.ljp[S.ti * md.ntype + ions.ts[e.x]], p, Sv);
+  const double fs = fma(S.qi * ions.ws[e.x], pair_poly(fx.ii[p.idx], p), lj);
   pair_add(fx, fs, dx, dy, dz, A.l);
 }
 
@@ -578,8 +579,8 @@ __device__ __forceinline__ void pair_ion_ele_fix(const PairSite &S, const CellsD
     return;
   }
   const PairArg p = pair_arg(Sv);
-  double fs = S.qi * Q[eles.order[e.x]] * pair_poly(fx.ie[p.idx], p);
-  if (md.ntype) fs += pair_lj(md.ljp[S.ti * md.ntype + (md.ntype - 1)], p, Sv);
+  const double lj = md.ntype ? pair_lj(md.ljp[S.ti * md.ntype + (md.ntype - 1)], p, Sv) : 0.0;
+  const double fs = fma(S.qi * Q[eles.order[e.x]], pair_poly(fx.ie[p.idx], p), lj);
   pair_add(fx, fs, dx, dy, dz, A.l);
 }
 
@@ -851,7 +852,7 @@ k_electrode_rhs(int64_t ne, const double *__restrict__ ex, const double *__restr
   } else if (!F32) {
     for (int k = lane; k < K; k += 32) {
       double cs, sn;
-      sincos_turns(phase64(__ldg(&modes[k]), ux, uy, uz), tab, cs, sn);
+      sincos_turns_fix(phase64(__ldg(&modes[k]), ux, uy, uz), tab, cs, sn);
       const double2 cf = __ldg(&coefS[k]);
       acc = fma(-cf.x, cs, acc);
       acc = fma(-cf.y, sn, acc);
@@ -1443,7 +1444,7 @@ k_ion_forces(int64_t ni, CellsDev ions, CellsDev eles, ListsDev nl, const double
              double3 invL, float3 kvf, double Lx, double Ly, double alpha, double eta, double rc, double slab,
              ForceF32 pf, const double *__restrict__ scal, MdDev md, const double *__restrict__ x_orig,
              const double *__restrict__ y_orig, const double *__restrict__ z_orig, double *__restrict__ F,
-             double *__restrict__ epart, const float4 *__restrict__ Fii, PairFix fx) {
+             double *__restrict__ epart, const float4 *__restrict__ Fii, PairFix fx, const double *__restrict__ kv) {
   static_assert(PART == 0 || (PART == 2 && F32 && !EN), "the split force pass is the mixed form's, without energies");
   __shared__ double red[kWarpsPerBlock][4];
   __shared__ int2 wq[kWarpsPerBlock][64];
@@ -1480,13 +1481,16 @@ k_ion_forces(int64_t ni, CellsDev ions, CellsDev eles, ListsDev nl, const double
       for (int k = lane; k < K; k += 32) {
         const int4 m = __ldg(&modes[k]);
         double cs, sn;
-        sincos_turns(phase64(m, ux, uy, uz), tab, cs, sn);
+        sincos_turns_fix(phase64(m, ux, uy, uz), tab, cs, sn);
         const double2 cf = __ldg(&coefF[k]);
         const double im = fma(cf.x, cs, -cf.y * sn);
-        fk[0] = fma(tpx * m.x, im, fk[0]);
-        fk[1] = fma(tpy * m.y, im, fk[1]);
-        fk[2] = fma(tpz * m.z, im, fk[2]);
+        fk[0] = fma(__ldg(kv + k), im, fk[0]);
+        fk[1] = fma(__ldg(kv + K + k), im, fk[1]);
+        fk[2] = fma(__ldg(kv + 2 * K + k), im, fk[2]);
       }
+      fk[0] *= tpx;
+      fk[1] *= tpy;
+      fk[2] *= tpz;
     } else {
       const uint32_t vx = (uint32_t)(ux >> 32), vy = (uint32_t)(uy >> 32), vz = (uint32_t)(uz >> 32);
       for (int k = lane; k < K; k += 32) {
@@ -1923,7 +1927,7 @@ void ion_forces(srbe_ctx *c, bool energies) {
     kern<<<nblk, kGatherThreads, 0, c->stream>>>(c->ni, ions, eles, lists_dev(c), c->Q.p, c->Q32.p, K, c->dm.p, coef,
                                                  c->coef32.p, c->tab.p, invL, kvf, c->L[0], c->L[1], c->alpha, c->eta,
                                                  c->rc, slab, pf, c->scal.p, md, c->x.p, c->y.p, c->z.p, c->F.p, ep,
-                                                 part2 ? c->fii.p : nullptr, pair_fix(c));
+                                                 part2 ? c->fii.p : nullptr, pair_fix(c), c->kv.p);
     c->launches++;
     c->mode_evals += c->ni * (int64_t)K;
   }

@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "../../include/srbe.h"
+#include "fixphase.cuh"
 
 namespace srbe {
 
@@ -266,6 +267,7 @@ struct srbe_ctx {
   srbe::DevBuf<double> mpart;                  // dipole partials [chunks]
   srbe::DevBuf<double2> coef;                  // per-mode c_k S(k) coefficients [K]
   srbe::DevBuf<float2> coef32;                 // their FP32 copy (mixed form)
+  srbe::DevBuf<double> kv;                     // the modes as doubles [3][K] (the FP64 form's force gather)
   srbe::DevBuf<float> Q32;                     // FP32 copy of the charges (mixed form)
   srbe::DevBuf<float2> lj32;                   // FP32 (sigma^2, eps) table (mixed form)
   srbe::DevBuf<double> scal;                   // device scalars (see kScal* indices)
@@ -385,6 +387,29 @@ __device__ __forceinline__ void sincos_turns(uint64_t th, const double2 *__restr
   const double2 T = __ldg(&tab[idx]);
   c = fma(T.x, cm1, fma(-T.y, sx, T.x));
   s = fma(T.y, cm1, fma(T.x, sx, T.y));
+}
+
+// The same in the FP64 form's per-step sums (structure factors, b, force gather): the remainder x gives
+// cos x - 1 and sin x in integer arithmetic (fixphase.cuh), which leaves the four FP64 multiply-adds of the
+// angle addition; the function above needs twelve FP64 operations, 7 clocks of an SM.  The rms error is
+// 4.66e-17 either way (table and roundings).  The set-up of A and the lattice phases, a few evaluations
+// per step at most, keep the function above and so A's bits.
+__device__ __forceinline__ void sincos_turns_fix(uint64_t th, const double2 *__restrict__ tab, double &c, double &s) {
+  const uint64_t t = th + (1ull << 53);
+  const unsigned idx = (unsigned)(t >> 54);
+  const int64_t rem = (int64_t)(th - ((uint64_t)idx << 54));     // in [-2^53, 2^53)
+  double cm1, sx;
+  small_cos_sin(rem, cm1, sx);
+  const double2 T = __ldg(&tab[idx]);
+  c = fma(T.x, cm1, fma(-T.y, sx, T.x));
+  s = fma(T.y, cm1, fma(T.x, sx, T.y));
+}
+
+// mode k's integer vector as doubles (SoA), so that the gather over ions needs no conversions
+__device__ __forceinline__ void store_mode(double *kv, int K, int k, int4 m) {
+  kv[k] = (double)m.x;
+  kv[K + k] = (double)m.y;
+  kv[2 * K + k] = (double)m.z;
 }
 
 // FP32 form: phase in turns from 32-bit fixed point (top half), reduced to [-pi, pi).
