@@ -1952,6 +1952,7 @@ int srbe_get_solver_stats(srbe_ctx *c, int *iterations, double *rel_residual) {
 namespace {
 void mlp_alloc(srbe_ctx *c) {
   const size_t n = (size_t)mlp_param_count();
+  c->mlp.split_ready = false;
   c->mlp.P.ensure(n);
   c->mlp.m1.ensure(n);
   c->mlp.m2.ensure(n);

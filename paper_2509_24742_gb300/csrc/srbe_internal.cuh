@@ -125,6 +125,8 @@ struct MlpState {
   bool ready = false;
   int t = 0;
   DevBuf<float> P, m1, m2, gpart, grad, D, data_D, data_T;
+  DevBuf<uint16_t> split;            // W1, W2 as blocked BF16 (hi, lo) operands of the forward pass
+  bool split_ready = false;          // false once the parameters have changed
   DevBuf<float> act;                 // activations of a training pass, row-major
   DevBuf<double> lpart, loss;        // squared errors: per split, per minibatch of an epoch
   DevBuf<double2> Slow;

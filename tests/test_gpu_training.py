@@ -71,6 +71,19 @@ def test_training_matches_oracle_steps(ctx, n, batch):
     assert abs(loss - ref_loss) < 1e-4 * ref_loss
 
 
+@pytest.mark.parametrize("n", [1, 127, 128, 129, 128 * 152, 128 * 152 + 1, 128 * 456 + 5])
+def test_prediction_at_tile_edges_matches_oracle(ctx, n):
+    """One row, partial tiles, one tile per SM, the first tile of the second group of warps, several tiles
+    per group.  The products keep 16 significand bits (split BF16), 1.5e-5 per term; 128 terms of random
+    sign leave about 1e-5 / sqrt(128) of the sum, so 1e-5 of the norm; new parameters are seen at once."""
+    D, _ = rows(n, 3 * n + 1)
+    for seed in (3, 4):
+        ctx.mlp_init(seed=seed)
+        y = ctx.mlp_predict(D)
+        ref = omlp.forward(ctx.mlp_params(), D)
+        assert np.linalg.norm(y - ref) < 1e-5 * np.linalg.norm(ref)
+
+
 def shuffles(n, epochs, seed):
     """Fisher-Yates rows of every epoch, one Philox4x64-10 word per exchange."""
     out, ctr = [], 0
