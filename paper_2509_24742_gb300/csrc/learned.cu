@@ -27,37 +27,47 @@ constexpr int kNtrain = oXm;     // trainable entries come first
 
 __device__ __forceinline__ float silu(float z) { return __fdividef(z, 1.f + __expf(-z)); }
 
-// S_low[m] = sum_i q_i exp(i 2 pi m z_i / L_z), m = 1..8, one block, fixed order
-__global__ void k_low_modes(int64_t n, const double *__restrict__ z, const double *__restrict__ q, double invLz,
-                            double2 *__restrict__ S) {
-  __shared__ double red[2 * kNlow][256];
-  const int t = threadIdx.x;
+// S_low[m] = sum_i q_i exp(i 2 pi m z_i / L_z), m = 1..8: one partial per block of 256 ions (Re, Im of
+// the 8 modes), added in block order by the descriptors.  (One block over all ions: 98 us at 8,000.)
+constexpr int kLowBlocks = 64;
+__global__ void __launch_bounds__(256)
+k_low_modes(int64_t n, const double *__restrict__ z, const double *__restrict__ q, double invLz,
+            double *__restrict__ part) {
+  __shared__ double red[8][2 * kNlow];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   double a[2 * kNlow];
+#pragma unroll
   for (int m = 0; m < 2 * kNlow; ++m) a[m] = 0.0;
-  for (int64_t i = t; i < n; i += 256) {
+  for (int64_t i = (int64_t)blockIdx.x * 256 + t; i < n; i += (int64_t)gridDim.x * 256) {
     const uint64_t u = to_turns64(z[i], invLz);
+    const double w = q[i];
+#pragma unroll
     for (int m = 0; m < kNlow; ++m) {
       float c, s;
       sincos_turns32((uint32_t)((u * (uint64_t)(m + 1)) >> 32), c, s);
-      a[2 * m] += q[i] * c;
-      a[2 * m + 1] += q[i] * s;
+      a[2 * m] += w * c;
+      a[2 * m + 1] += w * s;
     }
   }
-  for (int m = 0; m < 2 * kNlow; ++m) red[m][t] = a[m];
-  __syncthreads();
-  for (int s = 128; s > 0; s >>= 1) {
-    if (t < s)
-      for (int m = 0; m < 2 * kNlow; ++m) red[m][t] += red[m][t + s];
-    __syncthreads();
+#pragma unroll
+  for (int m = 0; m < 2 * kNlow; ++m) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) a[m] += __shfl_xor_sync(0xffffffffu, a[m], o);
+    if (lane == 0) red[warp][m] = a[m];
   }
-  if (t < kNlow) S[t] = make_double2(red[2 * t][0], red[2 * t + 1][0]);
+  __syncthreads();
+  if (t < 2 * kNlow) {
+    double s = red[0][t];
+    for (int w = 1; w < 8; ++w) s += red[w][t];
+    part[blockIdx.x * 2 * kNlow + t] = s;
+  }
 }
 
 // descriptors, one warp per electrode site; lane b owns basis function b
 __global__ void __launch_bounds__(256)
 k_descriptors(int64_t ne, const double *__restrict__ ex, const double *__restrict__ ey, const double *__restrict__ ez,
               const float4 *__restrict__ ion_pf, const int32_t *__restrict__ ei, const int32_t *__restrict__ ei_n,
-              int cap, float Lx, float Ly, float rc2, const double2 *__restrict__ Slow, double invLz,
+              int cap, float Lx, float Ly, float rc2, const double2 *__restrict__ low, int nlow, double invLz,
               float *__restrict__ D) {
   const int lane = threadIdx.x & 31;
   const int64_t j = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -98,7 +108,13 @@ k_descriptors(int64_t ne, const double *__restrict__ ex, const double *__restric
     const uint64_t u = to_turns64(ez[j], invLz);
     float c, s;
     sincos_turns32((uint32_t)((u * (uint64_t)(lane + 1)) >> 32), c, s);
-    const double2 S = Slow[lane];
+    double2 S = make_double2(0.0, 0.0);
+#pragma unroll 8
+    for (int b = 0; b < nlow; ++b) {
+      const double2 v = __ldg(low + b * kNlow + lane);
+      S.x += v.x;
+      S.y += v.y;
+    }
     row[64 + 2 * lane] = (float)(c * S.x + s * S.y);
     row[64 + 2 * lane + 1] = (float)(c * S.y - s * S.x);
   }
@@ -653,12 +669,14 @@ int mlp_input_width() { return kIn; }
 
 void mlp_descriptors(srbe_ctx *c, float *D_dev) {
   const int64_t ne = c->ne;
-  c->mlp.Slow.ensure(kNlow);
-  k_low_modes<<<1, 256, 0, c->stream>>>(c->ni, c->z.p, c->q.p, 1.0 / c->L[2], c->mlp.Slow.p);
+  const int nlow = (int)std::max<int64_t>(1, std::min<int64_t>(kLowBlocks, (c->ni + 255) / 256));
+  c->mlp.Slow.ensure(kNlow * kLowBlocks);
+  k_low_modes<<<nlow, 256, 0, c->stream>>>(c->ni, c->z.p, c->q.p, 1.0 / c->L[2],
+                                           reinterpret_cast<double *>(c->mlp.Slow.p));
   const float rc = (float)c->rc;
   k_descriptors<<<blocks_for(ne * 32, 256), 256, 0, c->stream>>>(
       ne, c->ex.p, c->ey.p, c->ez.p, c->icells.pf.p, c->nbr.ei.p, c->nbr.ei_n.p, c->nbr.cap, (float)c->L[0],
-      (float)c->L[1], rc * rc, c->mlp.Slow.p, 1.0 / c->L[2], D_dev);
+      (float)c->L[1], rc * rc, c->mlp.Slow.p, nlow, 1.0 / c->L[2], D_dev);
   c->launches += 2;
   SRBE_CUDA(cudaGetLastError());
 }
