@@ -261,7 +261,8 @@ int srbe_get_phase_times(srbe_ctx *ctx, double *ms, int64_t *count);
 /* In the mixed form PCG runs as iterative refinement: the FP64 residual dpsi d + b - A y decides
  * convergence (tol as above), and each correction comes from Jacobi-preconditioned CG on an FP32 copy
  * of A (formed once per electrode; half the bytes per product), in the Chronopoulos-Gear arrangement
- * (one grid-wide reduction per iteration), run until its residual has fallen by 1e-4; maxit bounds
+ * (one grid-wide reduction per iteration), run until its residual has fallen by 1e-4 or, once that is within
+ * 1e-5, to a quarter of the tolerance; maxit bounds
  * these inner iterations, which srbe_get_solver_stats counts.  The inner sums are FP32, so the
  * iteration count can differ by a few between builds that group them differently; the FP64 residual
  * bar does not.

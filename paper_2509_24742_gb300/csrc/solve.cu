@@ -253,6 +253,8 @@ __device__ __forceinline__ DF df_add_df(DF a, DF b) {
 // once per step from HBM, so each row is split over kSplitWarps warps (contiguous column segments)
 // to keep enough loads in flight; the segments' double-floats are combined in a fixed order.
 constexpr int kSplitWarps = 4;
+// (The streaming policy is right even where the matrix fits L2, 75 of 126 MB at 3,072 sites: read with the
+// normal one it pushes out the step's lists and vectors, 80 us per step instead of 70.)
 __global__ void __launch_bounds__(256)
 k_charges_split(int64_t n, const float2 *__restrict__ B, const float2 *__restrict__ b, double dpsi,
                 const double *__restrict__ qd, const float2 *__restrict__ we, double wd, double s_e,
@@ -526,6 +528,7 @@ struct PcgArgs {
   const float *A32;
   float *r32, *z32, *p32, *Ap32, *d32, *s32, *part32;
   const float *dinv32;
+  int srows;         // rows of A32 each block keeps in shared memory (0: none, the rows stream from L2)
 };
 
 __device__ double grid_dot_sum(const PcgArgs &a, double mine, int slot, cg::grid_group &grid) {
@@ -826,17 +829,200 @@ __device__ float grid_gemv32_dot(const PcgArgs &a, const float *u, float *w) {
   return dl;
 }
 
+// The inner solve for electrodes whose block rows nearly fit the shared memory (n a multiple of 4, at
+// most kCacheMaxN): every block keeps its first a.srows rows of A32 there for the whole solve (a 3,072-
+// site electrode has 20 or 21 rows of 12 KB per block, 18 fit), so that an inner iteration streams 5.6 MB
+// instead of 37.7 MB, and the elements of its rows live in registers of its first warp: u is the only
+// vector that is exchanged through memory.  What is left per iteration is two grid barriers, the load of
+// u and the reduction's partials, and 1 us of shared-memory reads.  3,072 sites: 8.9 us per iteration, 10.4 us
+// with rows streamed from L2 and the vectors in memory.
+constexpr int kPcgStaticSmem = 11264;      // bound of k_pcg_mixed's static shared memory
+constexpr int kCacheMaxN = 4096, kCacheVecs = kCacheMaxN / 4 / 8 / 32, kCacheMaxRows = 32;
+constexpr int kCacheGroup = 6, kCacheStream = 3;
+
+// eight sums over the warp: three exchanges halve the values a lane carries, two finish the lane's own
+// one; lane 4 i (and its three followers) ends with value i
+__device__ __forceinline__ float warp_sum8(const float *v, int lane) {
+  float a[4], b[2];
+  const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const float keep = h16 ? v[4 + k] : v[k], give = h16 ? v[k] : v[4 + k];
+    a[k] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
+  }
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const float keep = h8 ? a[2 + k] : a[k], give = h8 ? a[k] : a[2 + k];
+    b[k] = keep + __shfl_xor_sync(0xffffffffu, give, 8);
+  }
+  float c = (h4 ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, h4 ? b[0] : b[1], 4);
+  c += __shfl_xor_sync(0xffffffffu, c, 2);
+  c += __shfl_xor_sync(0xffffffffu, c, 1);
+  return c;
+}
+
+// (A32 u)[row] for thread t < number of this block's rows, row = blockIdx.x + t gridDim.x (0 elsewhere)
+__device__ float block_rows_cached(const PcgArgs &a, const float4 *sA, const float *u) {
+  __shared__ float part[8][kCacheMaxRows + 8];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int G = gridDim.x, n = (int)a.n, nv = n / 4, seg = (nv + 7) / 8, c0 = warp * seg, c1 = min(nv, c0 + seg);
+  const int nrow = (n - (int)blockIdx.x + G - 1) / G, cached = min(a.srows, nrow);
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  int col[kCacheVecs];
+  float4 uv[kCacheVecs], m[kCacheStream][kCacheVecs];
+#pragma unroll
+  for (int t = 0; t < kCacheVecs; ++t) {
+    const int j = c0 + lane + 32 * t;
+    uv[t] = j < c1 ? __ldcg(reinterpret_cast<const float4 *>(u) + j) : zero;
+    col[t] = j < c1 ? j : c0;                // a valid column; its u is zero
+  }
+  auto fetch = [&](int r0) {
+#pragma unroll
+    for (int k = 0; k < kCacheStream; ++k)
+#pragma unroll
+      for (int t = 0; t < kCacheVecs; ++t)
+        m[k][t] = r0 + k < nrow && 32 * t < seg
+                      ? __ldcg(reinterpret_cast<const float4 *>(a.A32 + (blockIdx.x + (int64_t)(r0 + k) * G) * n) + col[t])
+                      : zero;
+  };
+  auto put = [&](const float *v, int r0, int count) {
+    const float s = warp_sum8(v, lane);
+    if ((lane & 3) == 0 && (lane >> 2) < count) part[warp][r0 + (lane >> 2)] = s;
+  };
+  fetch(cached);
+  for (int r0 = 0; r0 < cached; r0 += kCacheGroup) {
+    float v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = 0.f;
+#pragma unroll
+    for (int k = 0; k < kCacheGroup; ++k) {
+      const float4 *row = sA + min(r0 + k, cached - 1) * nv;
+#pragma unroll
+      for (int t = 0; t < kCacheVecs; ++t)
+        if (32 * t < seg) v[k] += Vec<float>::dot(row[col[t]], uv[t]);
+    }
+    put(v, r0, min(kCacheGroup, cached - r0));
+  }
+  for (int r0 = cached; r0 < nrow; r0 += kCacheStream) {
+    float v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = 0.f;
+#pragma unroll
+    for (int k = 0; k < kCacheStream; ++k)
+#pragma unroll
+      for (int t = 0; t < kCacheVecs; ++t) v[k] += Vec<float>::dot(m[k][t], uv[t]);
+    if (r0 + kCacheStream < nrow) fetch(r0 + kCacheStream);
+    put(v, r0, min(kCacheStream, nrow - r0));
+  }
+  __syncthreads();
+  float w = 0.f;
+  if ((int)threadIdx.x < nrow) {
+    w = part[0][threadIdx.x];
+#pragma unroll
+    for (int k = 1; k < 8; ++k) w += part[k][threadIdx.x];
+  }
+  __syncthreads();
+  return w;
+}
+
+// sums of the first warp's values over the grid (its other lanes hold zeros), the same on every thread
+__device__ float3 grid_sum3_warp0(const PcgArgs &a, float v0, float v1, float v2, int slot, cg::grid_group &grid) {
+  __shared__ float3 tot;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float *P = a.part32 + (size_t)slot * 3 * gridDim.x;
+  auto fold = [&] {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      v0 += __shfl_xor_sync(0xffffffffu, v0, o);
+      v1 += __shfl_xor_sync(0xffffffffu, v1, o);
+      v2 += __shfl_xor_sync(0xffffffffu, v2, o);
+    }
+  };
+  if (warp == 0) {
+    fold();
+    if (lane == 0) {
+      P[blockIdx.x] = v0;
+      P[gridDim.x + blockIdx.x] = v1;
+      P[2 * gridDim.x + blockIdx.x] = v2;
+    }
+  }
+  grid.sync();
+  if (warp == 0) {
+    v0 = v1 = v2 = 0.f;
+    for (unsigned b = lane; b < gridDim.x; b += 32) {
+      v0 += __ldcg(P + b);
+      v1 += __ldcg(P + gridDim.x + b);
+      v2 += __ldcg(P + 2 * gridDim.x + b);
+    }
+    fold();
+    if (lane == 0) tot = make_float3(v0, v1, v2);
+  }
+  __syncthreads();
+  return tot;
+}
+
+// one correction: solves A delta = r until the inner residual's square has fallen to stop, by the
+// Chronopoulos-Gear iteration of k_pcg_mixed, and adds delta to y.  (The pipelined form with one barrier
+// per iteration does not reach 1e-4 with FP32 products: its recurrences for A-products drift.)
+__device__ void pcg_inner_cached(const PcgArgs &a, const float4 *sA, float stop, int &it, int &fslot,
+                                 cg::grid_group &grid) {
+  const int64_t row = blockIdx.x + (int64_t)threadIdx.x * gridDim.x;
+  const bool mine = threadIdx.x < 32 && row < a.n;      // rows per block <= 32: the first warp owns them
+  float r = 0.f, u = 0.f, x = 0.f, p = 0.f, s = 0.f, dv = 0.f;
+  if (mine) {
+    dv = a.dinv32[row];
+    r = (float)__ldcg(a.r + row);
+    u = dv * r;
+    a.z32[row] = u;
+  }
+  grid.sync();
+  float w = block_rows_cached(a, sA, a.z32);
+  float3 t = grid_sum3_warp0(a, r * u, w * u, r * r, fslot, grid);
+  fslot ^= 1;
+  float gamma = t.x, alpha = t.x / t.y, beta = 0.f;
+  float rrc = t.z;
+  while (it < a.maxit && rrc > stop) {
+    if (mine) {
+      p = fmaf(beta, p, u);
+      s = fmaf(beta, s, w);
+      x = fmaf(alpha, p, x);
+      r = fmaf(-alpha, s, r);
+      u = dv * r;
+      a.z32[row] = u;
+    }
+    grid.sync();
+    w = block_rows_cached(a, sA, a.z32);
+    t = grid_sum3_warp0(a, r * u, w * u, r * r, fslot, grid);
+    fslot ^= 1;
+    beta = t.x / gamma;
+    alpha = t.x / (t.y - beta * t.x / alpha);
+    gamma = t.x;
+    rrc = t.z;
+    ++it;
+  }
+  if (mine) a.y[row] += (double)x;
+}
+
 // The mixed form's iterative solve: iterative refinement in FP64 around Jacobi-PCG in FP32.  Each
 // outer pass forms the FP64 residual r = dpsi d + b - A y with A in FP64 and stops once
 // ||r|| <= tol ||dpsi d + b||; otherwise it solves A delta = r on an FP32 copy of A until the inner
-// residual has fallen by 1e-4, and adds delta to y in FP64.  The inner solve is the Chronopoulos-Gear
+// residual has fallen by 1e-4 (or to a quarter of the tolerance), and adds delta to y in FP64.  The inner solve is the Chronopoulos-Gear
 // form of preconditioned CG (Chronopoulos and Gear, J. Comput. Appl. Math. 25, 1989): it applies A to
 // the preconditioned residual u = M^-1 r and updates A p by the recurrence s = w + beta s, so the three
 // inner products of an iteration, (r, u), (A u, u) and (r, r), share one grid barrier; an iteration
 // costs two grid barriers instead of four.  maxit bounds the inner iterations over all passes; the
 // iteration count reported is theirs.  Q and psi_bar follow from Eqs. 9-10 as in k_pcg.
 __global__ void __launch_bounds__(256, 1) k_pcg_mixed(PcgArgs a) {
+  extern __shared__ __align__(16) float4 sA[];
   cg::grid_group grid = cg::this_grid();
+  if (a.srows) {
+    // this block's first rows of A32, read by every inner iteration (visible after the barriers below)
+    const int nv = (int)a.n / 4;
+    for (int r = 0; r < a.srows && blockIdx.x + (int64_t)r * gridDim.x < a.n; ++r) {
+      const float4 *src = reinterpret_cast<const float4 *>(a.A32 + (blockIdx.x + (int64_t)r * gridDim.x) * a.n);
+      for (int j = threadIdx.x; j < nv; j += blockDim.x) sA[r * nv + j] = __ldg(src + j);
+    }
+  }
   const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, gs = (int64_t)gridDim.x * blockDim.x;
   int slot = 0, fslot = 0;
   double vv = 0.0;
@@ -849,19 +1035,32 @@ __global__ void __launch_bounds__(256, 1) k_pcg_mixed(PcgArgs a) {
   slot = (slot + 1) & 7;            // its grid barrier also orders the writes of p before the products below
   int it = 0;
   bool converged = false;
+  double rr = 0.0;
+  bool fresh = false;               // rr is the squared residual of y as it stands
   float *x = a.d32, *r = a.r32, *u = a.z32, *w = a.Ap32, *p = a.p32, *s = a.s32;
   for (int outer = 0; outer < 16; ++outer) {
     grid_gemv(a, a.y, a.p, a.r, true);
     grid.sync();
-    double rr = 0.0;
+    rr = 0.0;
     for (int64_t i = gt; i < a.n; i += gs) rr += a.r[i] * a.r[i];
     rr = grid_dot_sum(a, rr, slot, grid);
     slot = (slot + 1) & 7;
+    fresh = true;
     if (rr <= a.tol2 * vv) {
       converged = true;
       break;
     }
     if (it >= a.maxit) break;
+    // the inner residual's target: 1e-4 of the outer one, but no less than a quarter of the tolerance, and
+    // that directly where it is at most 1e-5 away (a further correction would mostly overshoot it)
+    const double goal = 0.0625 * a.tol2 * vv;
+    const float stop = (float)(goal >= 1e-10 * rr ? goal : 1e-8 * rr);
+    if (a.srows) {
+      pcg_inner_cached(a, sA, stop, it, fslot, grid);
+      fresh = false;
+      grid.sync();
+      continue;
+    }
     // inner FP32 solve of A delta = r (delta in x)
     float gam = 0.f, rr32 = 0.f;
     for (int64_t i = gt; i < a.n; i += gs) {
@@ -879,7 +1078,6 @@ __global__ void __launch_bounds__(256, 1) k_pcg_mixed(PcgArgs a) {
     float3 t = grid_sum3f(a, gam, dl, rr32, fslot, grid);
     fslot ^= 1;
     float gamma = t.x, alpha = t.x / t.y, beta = 0.f;
-    const float stop = (float)(1e-8 * rr);   // inner residual 1e-4 of the outer one
     float rrc = t.z;
     while (it < a.maxit && rrc > stop) {
       gam = 0.f;
@@ -907,23 +1105,25 @@ __global__ void __launch_bounds__(256, 1) k_pcg_mixed(PcgArgs a) {
       ++it;
     }
     for (int64_t i = gt; i < a.n; i += gs) a.y[i] += (double)x[i];
+    fresh = false;
     grid.sync();
   }
-  // true residual, neutrality projection and psi_bar (Eqs. 9-10)
-  grid_gemv(a, a.y, a.p, a.r, true);
-  grid.sync();
-  double r2 = 0.0, ey = 0.0;
-  for (int64_t i = gt; i < a.n; i += gs) {
-    r2 += a.r[i] * a.r[i];
-    ey += a.y[i];
+  // neutrality projection and psi_bar (Eqs. 9-10).  The last pass's residual is that of y unless the
+  // passes ran out (y has moved since): only then is it formed once more.
+  double r2 = rr, ey = 0.0;
+  if (!fresh) {
+    grid_gemv(a, a.y, a.p, a.r, true);
+    grid.sync();
+    r2 = 0.0;
+    for (int64_t i = gt; i < a.n; i += gs) r2 += a.r[i] * a.r[i];
+    r2 = grid_dot_sum(a, r2, slot, grid);
+    slot = (slot + 1) & 7;
   }
-  r2 = grid_dot_sum(a, r2, slot, grid);
-    slot = (slot + 1) & 7;
+  for (int64_t i = gt; i < a.n; i += gs) ey += __ldcg(a.y + i);
   ey = grid_dot_sum(a, ey, slot, grid);
-    slot = (slot + 1) & 7;
   const double psi = -ey / a.s_e;
   for (int64_t i = gt; i < a.n; i += gs) {
-    const double q = fma(psi, a.we[i], a.y[i]);
+    const double q = fma(psi, a.we[i], __ldcg(a.y + i));
     a.Q[i] = q;
     a.Q32[i] = (float)q;
   }
@@ -945,7 +1145,7 @@ __global__ void k_to_float_n(int64_t n, const double *__restrict__ a, float *__r
 void charge_update_pcg(srbe_ctx *c) {
   const int64_t n = c->ne;
   const bool mixed = c->precision == SRBE_MIXED;
-  static int blocks_per_sm = 0, nsm = 0;
+  static int blocks_per_sm = 0, nsm = 0, smem_max = 0;
   if (!blocks_per_sm) {
     int dev = 0, b1 = 0, b2 = 0;
     SRBE_CUDA(cudaGetDevice(&dev));
@@ -954,6 +1154,9 @@ void charge_update_pcg(srbe_ctx *c) {
     SRBE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b2, k_pcg_mixed, 256, 0));
     blocks_per_sm = std::min(b1, b2);
     SRBE_REQUIRE(blocks_per_sm > 0, SRBE_ECUDA, "PCG kernel cannot be resident");
+    SRBE_CUDA(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    SRBE_CUDA(cudaFuncSetAttribute(k_pcg_mixed, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   smem_max - kPcgStaticSmem));
   }
   if (mixed && !c->pcg.a32_ready) {
     // the FP32 copy of A, formed once per electrode (outside any capture: the first pass after a
@@ -971,8 +1174,17 @@ void charge_update_pcg(srbe_ctx *c) {
     SRBE_CUDA(cudaGetLastError());
     c->pcg.a32_ready = true;
   }
-  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((n * 32 + 255) / 256, (int64_t)blocks_per_sm * nsm));
+  // mixed form up to 4,096 sites: one block per SM, as many of its rows of A32 in shared memory as fit
+  // beside the kernel's own 11 KB (above, and for n not a multiple of 4, every row streams from L2)
+  const bool cache = mixed && n % 4 == 0 && n <= kCacheMaxN;
+  const int most = cache ? nsm : blocks_per_sm * nsm;
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((n * 32 + 255) / 256, (int64_t)most));
+  const int64_t row_bytes = 4 * n, rows = (n + grid - 1) / grid;
+  const int srows = cache ? (int)std::min<int64_t>(rows, (int64_t)(smem_max - kPcgStaticSmem) / row_bytes) : 0;
+  const size_t smem = (size_t)srows * row_bytes;
+  SRBE_REQUIRE(!cache || rows <= kCacheMaxRows, SRBE_ESTATE, "too many rows per block for the cached product");
   PcgArgs a;
+  a.srows = srows;
   a.n = n;
   a.A = c->Amat.p;
   a.dinv = c->pcg.dinv.p;
@@ -1007,7 +1219,7 @@ void charge_update_pcg(srbe_ctx *c) {
   void *args[] = {&a};
   coop_before(c);
   SRBE_CUDA(cudaLaunchCooperativeKernel(mixed ? (const void *)k_pcg_mixed : (const void *)k_pcg, dim3(grid), dim3(256),
-                                        args, 0, c->stream));
+                                        args, smem, c->stream));
   coop_after(c);
   c->launches++;
 }
