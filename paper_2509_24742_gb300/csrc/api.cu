@@ -239,7 +239,8 @@ bool finite_all(const double *a, int64_t n) {
 
 // ---- staging kernels
 __global__ void k_deinterleave(int64_t n, const double *__restrict__ r, double Lx, double Ly, double *__restrict__ x,
-                               double *__restrict__ y, double *__restrict__ z) {
+                               double *__restrict__ y, double *__restrict__ z, double3 invL,
+                               uint64_t *__restrict__ iu) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   double X = r[3 * i], Y = r[3 * i + 1];
@@ -247,9 +248,14 @@ __global__ void k_deinterleave(int64_t n, const double *__restrict__ r, double L
   Y -= Ly * floor(Y / Ly);
   if (X >= Lx) X -= Lx;
   if (Y >= Ly) Y -= Ly;
+  const double Z = r[3 * i + 2];
   x[i] = X;
   y[i] = Y;
-  z[i] = r[3 * i + 2];
+  z[i] = Z;
+  // the ion structure factor's phase coordinates: once per ion here, not once per ion and mode tile there
+  iu[i] = to_turns64(X, invL.x);
+  iu[n + i] = to_turns64(Y, invL.y);
+  iu[2 * n + i] = to_turns64(Z, invL.z);
 }
 
 __global__ void k_site_turns(int64_t n, const double *__restrict__ x, const double *__restrict__ y,
@@ -645,11 +651,14 @@ void srbe_list_from_samples(srbe_ctx *c, const int32_t *samp, int P) {
 void forces_pass(srbe_ctx *c, bool energies, bool after_drift = false, bool check = true);
 
 // the captured step's mode list (K int4 + the step word) and weights, read from a mapped pinned slot
+// (and its step word once more into stepw: the next step's fused half kicks need it when dm holds theirs)
 __global__ void k_stage_modes(int K, const int4 *__restrict__ hm, const double *__restrict__ hw,
-                              int4 *__restrict__ dm, double *__restrict__ dc) {
+                              int4 *__restrict__ dm, double *__restrict__ dc, int4 *__restrict__ stepw) {
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k <= K; k += gridDim.x * blockDim.x) {
-    dm[k] = hm[k];
+    const int4 m = hm[k];
+    dm[k] = m;
     if (k < K) dc[k] = hw[k];
+    else *stepw = m;
   }
 }
 
@@ -683,6 +692,7 @@ struct DevSampleArgs {
   double L[3], G, V;
   int4 *dm;                 // modes: I at [0, M) (left as they are), samples at [M, M + P), step word at M + P
   double *dc;               // weights, the same layout
+  int4 *stepw;              // the step word once more (replayed steps), or null
   int *err;
 };
 __device__ __forceinline__ int cdf_search(const double *cdf, int n, double u) {
@@ -705,6 +715,7 @@ __global__ void __launch_bounds__(kSampleThreads) k_sample_exact(DevSampleArgs a
   if (t == 0) {
     s_count = 0;
     a.dm[a.M + a.P] = sw;   // the step word of the list (the thermostat reads its step half)
+    if (a.stepw) *a.stepw = sw;
   }
   const double *cd[3] = {a.cdf, a.cdf + 2 * a.sup[0] + 1, a.cdf + 2 * a.sup[0] + 1 + 2 * a.sup[1] + 1};
   __syncthreads();
@@ -750,7 +761,7 @@ inline int4 sample_word(uint64_t step, uint64_t seed) {
   return make_int4((int)(uint32_t)step, (int)(uint32_t)(step >> 32), (int)(uint32_t)seed, (int)(uint32_t)(seed >> 32));
 }
 
-DevSampleArgs dev_sample_args(srbe_ctx *c, const int4 *step_src) {
+DevSampleArgs dev_sample_args(srbe_ctx *c, const int4 *step_src, int4 *stepw = nullptr) {
   Extra *e = extra(c);
   DevSampleArgs a;
   a.step_src = step_src;
@@ -766,6 +777,7 @@ DevSampleArgs dev_sample_args(srbe_ctx *c, const int4 *step_src) {
   a.V = c->V;
   a.dm = c->dm.p;
   a.dc = c->dc.p;
+  a.stepw = stepw;
   a.err = e->dev_err.p;
   return a;
 }
@@ -793,32 +805,40 @@ void check_dev_sampler(srbe_ctx *c) {
   }
 }
 
-// one captured MD step of c; staged: the mode list is already on the device (batch graphs)
+// one captured MD step of c.  staged (batch graphs): the mode list is already on the device, and the step
+// is whole.  Otherwise the step leaves its closing half kick to the next replay or to integrate_close.
 void device_step(srbe_ctx *c, int slot, bool staged) {
   Extra *e = extra(c);
   const int K = c->K;
   SRBE_REQUIRE(c->dm.cap > (size_t)K && c->dc.cap >= (size_t)K && e->slot[slot].dhm, SRBE_ESTATE,
                "mode buffers not reserved for a captured step");
-  if (!staged) {
-    // the mode list comes in through a kernel on the side stream that reads the pinned slot while
-    // the opening kick runs (nothing before S1 reads it; the opening kick has no thermostat): the
-    // host's list, or with the device sampler only the slot's (step, seed) word
-    SRBE_CUDA(cudaEventRecord(c->ev_fork, c->stream));
-    SRBE_CUDA(cudaStreamWaitEvent(c->side, c->ev_fork, 0));
-    if (e->dev_sampler)
-      k_sample_exact<<<1, kSampleThreads, 0, c->side>>>(dev_sample_args(c, e->slot[slot].dhm + K));
-    else
-      k_stage_modes<<<std::min(blocks_for((int64_t)K + 1, 256), 64u), 256, 0, c->side>>>(K, e->slot[slot].dhm,
-                                                                                         e->slot[slot].dhw, c->dm.p,
-                                                                                         c->dc.p);
-    c->launches++;
-    SRBE_CUDA(cudaGetLastError());
-    SRBE_CUDA(cudaEventRecord(c->ev_modes, c->side));
+  if (staged) {
+    integrate_open(c);
+    forces_pass(c, false, true);
+    integrate_close(c);
+    return;
   }
-  integrate_kick_drift(c, 0.5 * c->dt, true);
-  if (!staged) SRBE_CUDA(cudaStreamWaitEvent(c->stream, c->ev_modes, 0));
+  SRBE_REQUIRE(c->stepw.cap >= 2, SRBE_ESTATE, "step words not reserved for a captured step");
+  // the mode list comes in through a kernel on the side stream that reads the pinned slot while the kick
+  // runs (nothing before S1 reads it, and the kick takes the step before's word from stepw): the host's
+  // list, or with the device sampler only the slot's (step, seed) word
+  SRBE_CUDA(cudaEventRecord(c->ev_fork, c->stream));
+  SRBE_CUDA(cudaStreamWaitEvent(c->side, c->ev_fork, 0));
+  if (e->dev_sampler)
+    k_sample_exact<<<1, kSampleThreads, 0, c->side>>>(dev_sample_args(c, e->slot[slot].dhm + K, c->stepw.p + slot));
+  else
+    k_stage_modes<<<std::min(blocks_for((int64_t)K + 1, 256), 64u), 256, 0, c->side>>>(
+        K, e->slot[slot].dhm, e->slot[slot].dhw, c->dm.p, c->dc.p, c->stepw.p + slot);
+  c->launches++;
+  SRBE_CUDA(cudaGetLastError());
+  SRBE_CUDA(cudaEventRecord(c->ev_modes, c->side));
+  integrate_close_open(c, c->stepw.p + (1 - slot));
+  SRBE_CUDA(cudaStreamWaitEvent(c->stream, c->ev_modes, 0));
   forces_pass(c, false, true);
-  integrate_kick_drift(c, 0.5 * c->dt, false);
+  // the closing half kick is now pending (any non-zero word); on the side stream, beside the force pass
+  SRBE_CUDA(cudaMemsetAsync(c->pending.p, 1, sizeof(int), c->side));
+  SRBE_CUDA(cudaEventRecord(c->ev_modes, c->side));
+  SRBE_CUDA(cudaStreamWaitEvent(c->stream, c->ev_modes, 0));
 }
 
 // one pass of the host-I/O force provider: mode list from the slot (side stream), positions from the
@@ -832,7 +852,7 @@ void provider_step(srbe_ctx *c, int slot) {
   SRBE_CUDA(cudaStreamWaitEvent(c->side, c->ev_fork, 0));
   k_stage_modes<<<std::min(blocks_for((int64_t)K + 1, 256), 64u), 256, 0, c->side>>>(K, e->slot[slot].dhm,
                                                                                      e->slot[slot].dhw, c->dm.p,
-                                                                                     c->dc.p);
+                                                                                     c->dc.p, c->stepw.p + slot);
   SRBE_CUDA(cudaEventRecord(c->ev_modes, c->side));
   uint64_t *iu = c->iu.ensure((size_t)3 * std::max<int64_t>(c->ni, 1));
   const double3 invL = make_double3(1.0 / c->L[0], 1.0 / c->L[1], 1.0 / c->L[2]);
@@ -852,6 +872,7 @@ void provider_step(srbe_ctx *c, int slot) {
 
 void ensure_slot_buffers(srbe_ctx *c) {
   Extra *e = extra(c);
+  c->stepw.ensure(2);
   SRBE_CUDA(cudaStreamSynchronize(c->stream));
   if (e->slot_cap < c->K) {
     for (auto &sl : e->slot) {
@@ -1024,7 +1045,7 @@ void charges_pass(srbe_ctx *c, bool after_drift) {
   SRBE_CUDA(cudaEventRecord(c->ev_join, c->side));
   phase_begin(c, kPhS1);
   structure_factor(c, c->ni, c->x.p, c->y.p, c->z.p, c->q.p, c->S1.p, nullptr, kScalMion, 0,
-                   after_drift ? c->iu.p : nullptr, c->q32.p);
+                   after_drift || c->iu_fresh ? c->iu.p : nullptr, c->q32.p);
   phase_end(c, kPhS1);
   SRBE_CUDA(cudaStreamWaitEvent(c->stream, c->ev_join, 0));
   phase_begin(c, kPhRhs);
@@ -1103,11 +1124,11 @@ void eager_step(srbe_ctx *c, uint64_t seed0) {
   c->md_step++;
   sample_into(c, seed0, c->md_step);
   phase_begin(c, kPhIntegrate);
-  integrate_kick_drift(c, 0.5 * c->dt, true);
+  integrate_open(c);
   phase_end(c, kPhIntegrate);
   forces_pass(c, false, true);
   phase_begin(c, kPhIntegrate);
-  integrate_kick_drift(c, 0.5 * c->dt, false);
+  integrate_close(c);
   phase_end(c, kPhIntegrate);
 }
 
@@ -1222,6 +1243,7 @@ int srbe_create(const double box[3], double alpha, double eta, double rc, int P,
     SRBE_CUDA(cudaHostGetDevicePointer((void **)&c->d_status, c->h_status, 0));
     c->scal.ensure(kScalCount);
     SRBE_CUDA(cudaMemsetAsync(c->scal.p, 0, sizeof(double) * kScalCount, c->stream));
+    SRBE_CUDA(cudaMemsetAsync(c->pending.ensure(1), 0, sizeof(int), c->stream));
     c->hx->sampler.init(c->L, c->alpha, c->M, c->mmax);
     c->G = c->hx->sampler.G();
   });
@@ -1377,8 +1399,10 @@ int srbe_set_positions(srbe_ctx *c, int64_t n_ion, const double *r, const double
       SRBE_CUDA(cudaMemcpyAsync(c->q.p, q, sizeof(double) * n_ion, cudaMemcpyHostToDevice, c->stream));
       k_to_f32<<<blocks_for(n_ion, 256), 256, 0, c->stream>>>(n_ion, c->q.p, c->q32.ensure(n));
       c->launches++;
-      k_deinterleave<<<blocks_for(n_ion, 256), 256, 0, c->stream>>>(n_ion, aos, c->L[0], c->L[1], c->x.p, c->y.p,
-                                                                   c->z.p);
+      k_deinterleave<<<blocks_for(n_ion, 256), 256, 0, c->stream>>>(
+          n_ion, aos, c->L[0], c->L[1], c->x.p, c->y.p, c->z.p,
+          make_double3(1.0 / c->L[0], 1.0 / c->L[1], 1.0 / c->L[2]), c->iu.ensure(3 * n));
+      c->iu_fresh = true;
       c->launches++;
       SRBE_CUDA(cudaGetLastError());
     }
@@ -1406,8 +1430,10 @@ int srbe_set_positions_dev(srbe_ctx *c, int64_t n_ion, const double *r_dev, cons
       SRBE_CUDA(cudaMemcpyAsync(c->q.p, q_dev, sizeof(double) * n_ion, cudaMemcpyDeviceToDevice, c->stream));
       k_to_f32<<<blocks_for(n_ion, 256), 256, 0, c->stream>>>(n_ion, c->q.p, c->q32.ensure(n));
       c->launches++;
-      k_deinterleave<<<blocks_for(n_ion, 256), 256, 0, c->stream>>>(n_ion, r_dev, c->L[0], c->L[1], c->x.p, c->y.p,
-                                                                   c->z.p);
+      k_deinterleave<<<blocks_for(n_ion, 256), 256, 0, c->stream>>>(
+          n_ion, r_dev, c->L[0], c->L[1], c->x.p, c->y.p, c->z.p,
+          make_double3(1.0 / c->L[0], 1.0 / c->L[1], 1.0 / c->L[2]), c->iu.ensure(3 * n));
+      c->iu_fresh = true;
       c->launches++;
       SRBE_CUDA(cudaGetLastError());
     }
@@ -1797,24 +1823,38 @@ int srbe_step(srbe_ctx *c, int nsteps, uint64_t seed0) {
       }
     }
     if (graphs && !e->graph_failed) {
-      for (int s = 0; s < nsteps; ++s) {
-        report_status(c, false); // what the host sees so far (no wait)
-        c->md_step++;
-        const int slot = (int)(c->md_step & 1);
-        if (e->dev_sampler) {
-          // the captured step samples its modes on the device from this word
-          SRBE_CUDA(cudaEventSynchronize(e->slot[slot].done));
-          e->slot[slot].hm[c->K] = sample_word(c->md_step, seed0);
-        } else {
-          build_host_list(c, seed0, c->md_step);
-          fill_slot(c, slot);
+      int queued = 0;
+      // a replayed step leaves its closing half kick to the next one: the last is closed here, also when
+      // the run ends early
+      auto close = [&] {
+        if (queued) integrate_close(c);
+        queued = 0;
+      };
+      try {
+        for (int s = 0; s < nsteps; ++s) {
+          report_status(c, false); // what the host sees so far (no wait)
+          c->md_step++;
+          const int slot = (int)(c->md_step & 1);
+          if (e->dev_sampler) {
+            // the captured step samples its modes on the device from this word
+            SRBE_CUDA(cudaEventSynchronize(e->slot[slot].done));
+            e->slot[slot].hm[c->K] = sample_word(c->md_step, seed0);
+          } else {
+            build_host_list(c, seed0, c->md_step);
+            fill_slot(c, slot);
+          }
+          coop_before(c);
+          SRBE_CUDA(cudaGraphLaunch(e->slot[slot].exec, c->stream));
+          ++queued;
+          coop_after(c);
+          SRBE_CUDA(cudaEventRecord(e->slot[slot].done, c->stream));
+          c->launches += e->graph_kernels;
         }
-        coop_before(c);
-        SRBE_CUDA(cudaGraphLaunch(e->slot[slot].exec, c->stream));
-        coop_after(c);
-        SRBE_CUDA(cudaEventRecord(e->slot[slot].done, c->stream));
-        c->launches += e->graph_kernels;
+      } catch (...) {
+        close();
+        throw;
       }
+      close();
       return;
     }
     for (int s = 0; s < nsteps; ++s) {
@@ -2263,6 +2303,7 @@ void snapshot_io(srbe_ctx *c, Snapshot &sn, bool save) {
   } else {
     c->md_step = sn.md_step;
     extra(c)->forces_valid = sn.forces_valid;
+    c->iu_fresh = false;
     neighbor_force_rebuild(c);
   }
 }

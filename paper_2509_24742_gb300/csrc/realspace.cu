@@ -1288,11 +1288,14 @@ __global__ void __launch_bounds__(256, 4) k_neighbor_update(NbrKernelArgs a) {
   }
 }
 
+__global__ void k_force_rebuild(int *flag) { flag[0] = flag[1] = 1; }
+
+// the next neighbour update rebuilds (queued behind the context's work: a copy from the host's stack
+// would have to be waited for)
 void neighbor_force_rebuild(srbe_ctx *c) {
-  int *f = c->nbr.flag.ensure(3);
-  const int one[2] = {1, 1};
-  SRBE_CUDA(cudaMemcpyAsync(f, one, sizeof(one), cudaMemcpyHostToDevice, c->stream));
-  SRBE_CUDA(cudaStreamSynchronize(c->stream));
+  k_force_rebuild<<<1, 1, 0, c->stream>>>(c->nbr.flag.ensure(3));
+  c->launches++;
+  SRBE_CUDA(cudaGetLastError());
 }
 
 void neighbor_update(srbe_ctx *c) {
@@ -1364,7 +1367,10 @@ void neighbor_update(srbe_ctx *c) {
     SRBE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, k_neighbor_update, 256, 0));
     SRBE_REQUIRE(blocks_per_sm > 0, SRBE_ECUDA, "neighbor-update kernel cannot be resident");
   }
-  const int want = (int)std::max<int64_t>(1, std::min<int64_t>((std::max<int64_t>(n, c->ne) * 32 + 255) / 256,
+  // one warp per list (ion-ion, ion-electrode, electrode-ion) as far as the blocks can be resident: in a
+  // small system the lists are then built side by side (400 ions + 384 sites: the rebuild takes 41 us, 47
+  // with a warp per ion)
+  const int want = (int)std::max<int64_t>(1, std::min<int64_t>(((2 * n + c->ne) * 32 + 255) / 256,
                                                                  (int64_t)blocks_per_sm * nsm));
   k_nbr_refresh<<<blocks_for(4 * std::max<int64_t>(n, 1), 128), 128, 0, c->stream>>>(a);
   SRBE_CUDA(cudaGetLastError());
@@ -2012,6 +2018,13 @@ __device__ __forceinline__ double wrap_periodic(double X, double L) {
   return X;
 }
 
+// A step opens with a half kick and the drift and closes with a half kick and the thermostat.  Inside a
+// run of replayed steps the closing half kick of one step and the opening of the next are one launch
+// (kBoth: the same operations in the same order, so the same bits): `pending` says whether the step before
+// left its closing half kick undone; the run's last one is closed by a launch of its own (kClose).
+// Separate launches took 4.7 + 4.4 us per step of the 11,072-site slab, one takes 5.4 us.
+enum { kClose = 0, kOpen = 1, kBoth = 2 };
+
 // The closing half kick (status != nullptr) also checks the step's forces and charges: a non-finite
 // F of this thread's ion or Q of the electrode site with the same index raises the context's flag.
 // One thread per (ion, component): the FP64 update of a component is a short dependent chain, and
@@ -2019,13 +2032,20 @@ __device__ __forceinline__ double wrap_periodic(double X, double L) {
 // per ion shorten the kernel's critical path.  blockIdx.y is the component (0 x, 1 y, 2 z).  Each
 // thread draws the same Philox words for its ion and forms its own one of the three normals (the
 // arithmetic of each component is unchanged: the results are the same bits as one thread per ion).
+template <int MODE>
 __global__ void k_kick_drift(int64_t n, double *__restrict__ x, double *__restrict__ y, double *__restrict__ z,
                              double *__restrict__ vx, double *__restrict__ vy, double *__restrict__ vz,
                              const double *__restrict__ F, const double *__restrict__ minv, double fac, double dt,
-                             int drift, double Lx, double Ly, Thermo th, double3 invL, uint64_t *__restrict__ iu,
-                             int64_t ne, const double *__restrict__ Q, int *__restrict__ status) {
+                             double Lx, double Ly, Thermo th, double3 invL, uint64_t *__restrict__ iu,
+                             int64_t ne, const double *__restrict__ Q, int *__restrict__ status,
+                             int *__restrict__ pending) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int d = blockIdx.y;
+  // the closing half kick (and its checks): always (kClose), never (kOpen), or if the step before has left
+  // it to this launch (kBoth)
+  const bool close = MODE == kClose || (MODE == kBoth && *pending != 0);
+  if (!close) status = nullptr;
+  if (MODE == kClose && i == 0 && d == 0) *pending = 0;
   if (d == 0 && status && i < ne && !isfinite(Q[i])) *(volatile int *)(status + kStatNonFiniteQ) = 1;
   if (i >= n) return;
   double *pos = d == 0 ? x : (d == 1 ? y : z);
@@ -2033,8 +2053,9 @@ __global__ void k_kick_drift(int64_t n, double *__restrict__ x, double *__restri
   const double w = fac * minv[i];
   const double f = F[d * n + i];
   if (status && !isfinite(f)) *(volatile int *)(status + kStatNonFiniteF) = 1;
-  double a = fma(w, f, vel[i]);
-  if (th.on) {
+  double a = vel[i];
+  if (close) a = fma(w, f, a);
+  if (close && th.on) {
     const int4 st = *th.step;
     const uint64_t step = (uint64_t)(uint32_t)st.x | ((uint64_t)(uint32_t)st.y << 32);
     uint64_t wd[4];
@@ -2064,8 +2085,9 @@ __global__ void k_kick_drift(int64_t n, double *__restrict__ x, double *__restri
     }
     a = fma(th.c1, a, g);
   }
+  if (MODE != kClose) a = fma(w, f, a);
   vel[i] = a;
-  if (drift) {
+  if (MODE != kClose) {
     double X = fma(dt, a, pos[i]);
     if (d < 2) X = wrap_periodic(X, d == 0 ? Lx : Ly);
     pos[i] = X;
@@ -2105,36 +2127,48 @@ void steepest_descent_move(srbe_ctx *c, double a, double dmax) {
   k_sd_move<<<blocks_for(c->ni, 256), 256, 0, c->stream>>>(c->ni, c->x.p, c->y.p, c->z.p, c->F.p, a, dmax, c->L[0],
                                                           c->L[1]);
   c->launches++;
+  c->iu_fresh = false;
   SRBE_CUDA(cudaGetLastError());
 }
 
-void integrate_kick_drift(srbe_ctx *c, double fac_kick, bool drift) {
+// which: kClose, kOpen or kBoth; step_word: device address of the step number the thermostat draws for
+static void kick(srbe_ctx *c, int which, const int4 *step_word) {
   if (c->ni == 0) return;
   Thermo th;
-  if (!drift && c->lang_gamma > 0.0) {
-    // the closing half kick of a step also applies the thermostat; the step number sits in dm[K]
-    SRBE_REQUIRE(c->dm.p && c->dm.cap > (size_t)c->K, SRBE_ESTATE, "mode list without its step word");
+  if (which != kOpen && c->lang_gamma > 0.0) {
+    // the closing half kick of a step also applies the thermostat
     th.on = 1;
     th.f32 = c->precision == SRBE_MIXED ? 1 : 0;
     th.c1 = std::exp(-c->lang_gamma * c->dt);
     th.s2 = (1.0 - th.c1 * th.c1) * kBoltz * c->lang_T;
     th.seed = c->lang_seed;
-    th.step = c->dm.p + c->K;
+    th.step = step_word;
   }
-  uint64_t *iu = drift ? c->iu.ensure((size_t)3 * c->ni) : nullptr;
+  uint64_t *iu = which != kClose ? c->iu.ensure((size_t)3 * c->ni) : nullptr;
   const double3 invL = make_double3(1.0 / c->L[0], 1.0 / c->L[1], 1.0 / c->L[2]);
   // the closing kick checks the step's forces and charges (one thread per ion and per site)
-  const int64_t ne = drift ? 0 : c->ne;
+  const int64_t ne = which == kOpen ? 0 : c->ne;
   const int64_t nt = std::max<int64_t>(c->ni, ne);
   // 64-thread blocks, one grid row per component: the FP64 arithmetic spreads over every SM even for
   // a few thousand ions
-  k_kick_drift<<<dim3(blocks_for(nt, 64), 3), 64, 0, c->stream>>>(c->ni, c->x.p, c->y.p, c->z.p, c->vx.p, c->vy.p,
-                                                         c->vz.p, c->F.p, c->minv.p, fac_kick, c->dt,
-                                                         drift ? 1 : 0, c->L[0], c->L[1], th, invL, iu, ne, c->Q.p,
-                                                         drift ? nullptr : c->d_status);
+  auto kern = which == kClose ? k_kick_drift<kClose> : (which == kOpen ? k_kick_drift<kOpen> : k_kick_drift<kBoth>);
+  kern<<<dim3(blocks_for(nt, 64), 3), 64, 0, c->stream>>>(c->ni, c->x.p, c->y.p, c->z.p, c->vx.p, c->vy.p, c->vz.p,
+                                                         c->F.p, c->minv.p, 0.5 * c->dt, c->dt, c->L[0], c->L[1], th,
+                                                         invL, iu, ne, c->Q.p, which == kOpen ? nullptr : c->d_status,
+                                                         c->pending.p);
   c->launches++;
   SRBE_CUDA(cudaGetLastError());
+  if (which != kClose) c->iu_fresh = true;
 }
+
+// the step number sits behind the mode list, in dm[K]
+void integrate_open(srbe_ctx *c) { kick(c, kOpen, nullptr); }
+void integrate_close(srbe_ctx *c) {
+  SRBE_REQUIRE(c->lang_gamma <= 0.0 || (c->dm.p && c->dm.cap > (size_t)c->K), SRBE_ESTATE,
+               "mode list without its step word");
+  kick(c, kClose, c->dm.p + c->K);
+}
+void integrate_close_open(srbe_ctx *c, const int4 *step_word) { kick(c, kBoth, step_word); }
 
 // non-finite check of the forces [3][nF / 3] and charges [nQ] of a pass outside the MD step
 __global__ void k_check_finite(int64_t nF, const double *__restrict__ F, int64_t nQ, const double *__restrict__ Q,

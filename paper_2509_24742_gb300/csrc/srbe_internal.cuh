@@ -211,7 +211,10 @@ struct srbe_ctx {
   srbe::DevBuf<uint64_t> eu;                   // fixed-point phase coordinates [3][ne], site order
   srbe::DevBuf<uint64_t> euw;                  // pair coordinates [3][ne], site order (FP64 form)
   srbe::DevBuf<float4> epf;                    // FP32 site positions (x, y, z, 0), site order
-  srbe::DevBuf<uint64_t> iu;                   // ion phase coordinates [3][ni] written by the drift of a step
+  srbe::DevBuf<uint64_t> iu;                   // ion phase coordinates [3][ni], written with the positions
+  bool iu_fresh = false;                       // they belong to the present positions
+  srbe::DevBuf<int> pending;                   // 1: the last replayed step's closing half kick is still to be done
+  srbe::DevBuf<int4> stepw;                    // step words of the last two replayed steps, by slot
   srbe::DevBuf<double> Bmat;                   // projected inverse J A^-1, ne x ne row-major
   srbe::DevBuf<float2> Bsplit;                 // its (hi, lo) FP32 split (mixed form)
   srbe::DevBuf<double> Amat;                   // A itself (kept for the refinement residual)
@@ -462,7 +465,9 @@ void mlp_grad_step(srbe_ctx *c, const float *D_dev, const float *T_dev, const in
 void ion_forces(srbe_ctx *c, bool energies);
 bool ion_forces_split(const srbe_ctx *c, bool energies);
 void ion_forces_ii(srbe_ctx *c);
-void integrate_kick_drift(srbe_ctx *c, double fac_kick, bool drift);
+void integrate_open(srbe_ctx *c);
+void integrate_close(srbe_ctx *c);
+void integrate_close_open(srbe_ctx *c, const int4 *step_word);
 void steepest_descent_move(srbe_ctx *c, double a, double dmax);
 void build_A_and_inverse(srbe_ctx *c);
 void energy_scalars(srbe_ctx *c);
