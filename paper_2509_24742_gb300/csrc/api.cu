@@ -514,7 +514,9 @@ void upload_table(srbe_ctx *c) {
 void reserve(srbe_ctx *c) {
   const int K = std::max(c->K, 1);
   int64_t ch;
-  const int64_t nch = std::max(sfac_chunks(c->ni, c->K, c->sf_occ, &ch), sfac_chunks(c->ne, c->K, c->sf_occ, &ch));
+  const bool f64 = c->precision == SRBE_FP64;
+  const int64_t nch =
+      std::max(sfac_chunks(c->ni, c->K, c->sf_occ, f64, &ch), sfac_chunks(c->ne, c->K, c->sf_occ, f64, &ch));
   c->partial.ensure((size_t)std::max<int64_t>(nch, 1) * K);
   c->mpart.ensure((size_t)std::max<int64_t>(nch, 1));
   c->coef.ensure((size_t)K);

@@ -492,7 +492,7 @@ void charge_residual(srbe_ctx *c, double *out_dev);
 void phase_begin(srbe_ctx *c, int ph);
 void phase_end(srbe_ctx *c, int ph);
 void reserve(srbe_ctx *c);
-int64_t sfac_chunks(int64_t n, int K, int occ, int64_t *chunk);
+int64_t sfac_chunks(int64_t n, int K, int occ, bool fp64, int64_t *chunk);
 
 inline unsigned blocks_for(int64_t n, int threads) { return (unsigned)((n + threads - 1) / threads); }
 
