@@ -325,18 +325,25 @@ __global__ void k_io_load(int64_t n, const double *__restrict__ r, double Lx, do
   iu[2 * n + i] = to_turns64(Z, invL.z);
 }
 
-// the force provider's output: F [3][ni] as [ni][3], Q and psi_bar into the caller's pinned buffers
+// the force provider's output: F [3][ni] as [ni][3], Q and psi_bar into the caller's pinned buffers; a
+// non-finite force or charge raises the context's flag (a check of its own was one more launch, 2.6 us)
 __global__ void k_io_store(int64_t ni, const double *__restrict__ F, double *__restrict__ Fo, int64_t ne,
                            const double *__restrict__ Q, double *__restrict__ Qo, const double *__restrict__ scal,
-                           double *__restrict__ psi) {
+                           double *__restrict__ psi, int *__restrict__ status) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < ni || i < ne; i += stride) {
     if (i < ni) {
-      Fo[3 * i] = F[i];
-      Fo[3 * i + 1] = F[ni + i];
-      Fo[3 * i + 2] = F[2 * ni + i];
+      const double fx = F[i], fy = F[ni + i], fz = F[2 * ni + i];
+      Fo[3 * i] = fx;
+      Fo[3 * i + 1] = fy;
+      Fo[3 * i + 2] = fz;
+      if (!(isfinite(fx) && isfinite(fy) && isfinite(fz))) *(volatile int *)(status + kStatNonFiniteF) = 1;
     }
-    if (i < ne && Qo) Qo[i] = Q[i];
+    if (i < ne) {
+      const double q = Q[i];
+      if (Qo) Qo[i] = q;
+      if (!isfinite(q)) *(volatile int *)(status + kStatNonFiniteQ) = 1;
+    }
     if (i == 0) *psi = scal[kScalPsi];
   }
 }
@@ -865,10 +872,10 @@ void provider_step(srbe_ctx *c, int slot) {
   SRBE_CUDA(cudaGetLastError());
   SRBE_CUDA(cudaStreamWaitEvent(c->stream, c->ev_modes, 0));
   forces_pass(c, false, true);
-  check_finite(c, true, true);
   const int64_t nt = std::max<int64_t>(std::max<int64_t>(c->ni, c->ne), 1);
   k_io_store<<<std::min(blocks_for(nt, 256), 304u), 256, 0, c->stream>>>(c->ni, c->F.p, e->io_dF, c->ne, c->Q.p,
-                                                                         e->io_dQ, c->scal.p, e->io_dpsi);
+                                                                         e->io_dQ, c->scal.p, e->io_dpsi,
+                                                                         c->d_status);
   c->launches++;
   SRBE_CUDA(cudaGetLastError());
 }
