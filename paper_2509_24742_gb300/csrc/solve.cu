@@ -1145,7 +1145,7 @@ __global__ void k_to_float_n(int64_t n, const double *__restrict__ a, float *__r
 void charge_update_pcg(srbe_ctx *c) {
   const int64_t n = c->ne;
   const bool mixed = c->precision == SRBE_MIXED;
-  static int blocks_per_sm = 0, nsm = 0, smem_max = 0;
+  static int blocks_per_sm = 0, nsm = 0;
   if (!blocks_per_sm) {
     int dev = 0, b1 = 0, b2 = 0;
     SRBE_CUDA(cudaGetDevice(&dev));
@@ -1154,9 +1154,6 @@ void charge_update_pcg(srbe_ctx *c) {
     SRBE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b2, k_pcg_mixed, 256, 0));
     blocks_per_sm = std::min(b1, b2);
     SRBE_REQUIRE(blocks_per_sm > 0, SRBE_ECUDA, "PCG kernel cannot be resident");
-    SRBE_CUDA(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    SRBE_CUDA(cudaFuncSetAttribute(k_pcg_mixed, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   smem_max - kPcgStaticSmem));
   }
   if (mixed && !c->pcg.a32_ready) {
     // the FP32 copy of A, formed once per electrode (outside any capture: the first pass after a
@@ -1175,14 +1172,21 @@ void charge_update_pcg(srbe_ctx *c) {
     c->pcg.a32_ready = true;
   }
   // mixed form up to 4,096 sites: one block per SM, as many of its rows of A32 in shared memory as fit
-  // beside the kernel's own 11 KB (above, and for n not a multiple of 4, every row streams from L2)
-  const bool cache = mixed && n % 4 == 0 && n <= kCacheMaxN;
+  // beside the kernel's own 11 KB (above, for n not a multiple of 4, and where the first warp's lanes are
+  // fewer than a block's rows, every row streams from L2)
+  const bool cache = mixed && n % 4 == 0 && n <= kCacheMaxN && (n + nsm - 1) / nsm <= kCacheMaxRows;
   const int most = cache ? nsm : blocks_per_sm * nsm;
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((n * 32 + 255) / 256, (int64_t)most));
-  const int64_t row_bytes = 4 * n, rows = (n + grid - 1) / grid;
-  const int srows = cache ? (int)std::min<int64_t>(rows, (int64_t)(smem_max - kPcgStaticSmem) / row_bytes) : 0;
-  const size_t smem = (size_t)srows * row_bytes;
-  SRBE_REQUIRE(!cache || rows <= kCacheMaxRows, SRBE_ESTATE, "too many rows per block for the cached product");
+  int srows = 0;
+  if (cache) {
+    int dev = 0, smem_max = 0;
+    SRBE_CUDA(cudaGetDevice(&dev));
+    SRBE_CUDA(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    SRBE_CUDA(cudaFuncSetAttribute(k_pcg_mixed, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   smem_max - kPcgStaticSmem));
+    srows = (int)std::min<int64_t>((n + grid - 1) / grid, (smem_max - kPcgStaticSmem) / (4 * n));
+  }
+  const size_t smem = (size_t)srows * 4 * n;
   PcgArgs a;
   a.srows = srows;
   a.n = n;
