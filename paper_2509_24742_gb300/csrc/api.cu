@@ -513,6 +513,10 @@ void upload_table(srbe_ctx *c) {
     const long double a = 2.0L * 3.141592653589793238462643383279502884L * (long double)j / (long double)kTab;
     h[j] = make_double2((double)cosl(a), (double)sinl(a));
   }
+  std::vector<longlong2> hi(kTab);
+  fix_table(hi.data());
+  SRBE_CUDA(cudaMemcpyAsync(c->tabi.ensure(kTab), hi.data(), sizeof(longlong2) * kTab, cudaMemcpyHostToDevice,
+                            c->stream));
   c->tab.ensure(kTab);
   SRBE_CUDA(cudaMemcpyAsync(c->tab.p, h.data(), sizeof(double2) * kTab, cudaMemcpyHostToDevice, c->stream));
   SRBE_CUDA(cudaStreamSynchronize(c->stream));

@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(kSfThreads)
 k_sfac_partial(int64_t n, const double *__restrict__ x, const double *__restrict__ y, const double *__restrict__ z,
                const uint64_t *__restrict__ u, const double *__restrict__ w, const float *__restrict__ w32, int K,
                const int4 *__restrict__ modes, double3 invL,
-               const double2 *__restrict__ tab, int64_t chunk, double2 *__restrict__ partial,
+               const longlong2 *__restrict__ tab, int64_t chunk, double2 *__restrict__ partial,
                double *__restrict__ mpart, SfFinish fin, int *__restrict__ done) {
   __shared__ uint64_t su[3][kSfThreads];
   __shared__ double sw[kSfThreads];
@@ -307,8 +307,8 @@ __global__ void k_sfac_reduce(SfFinish f) {
 // warp sums), which cost 64 cycles of a sub-partition each on this GPU, so longer chunks spread them
 // over more particles, while shorter ones give more blocks to hide latency with.  occ is a context
 // setting (default 8) that srbe_autotune_tiles / srbe_batch_autotune_tiles choose by timing.
-// The FP64 form is bound by the FP64 pipes (6 operations per particle and mode at 1.7 per clock and SM), so
-// while there are fewer than two blocks per SM its chunks shrink to 64 or 32 particles: 3,072 sites, 204
+// The FP64 form spends ten times as long on a particle, so while there are fewer than two blocks per SM its
+// chunks shrink to 64 or 32 particles: 3,072 sites, 204
 // modes (168 blocks, 16 SMs with two of them): 24.9 -> 18.4 us; 400 particles, 102 modes: 23.2 -> 12.3 us.
 int64_t sfac_chunks(int64_t n, int K, int occ, bool fp64, int64_t *chunk) {
   static int nsm = 0;
@@ -351,11 +351,11 @@ void structure_factor(srbe_ctx *c, int64_t n, const double *x, const double *y, 
     SRBE_REQUIRE(c->sfdone.cap >= (size_t)ktiles, SRBE_ESTATE, "tile counters not reserved for this size");
     dim3 grid((unsigned)nchunk, (unsigned)ktiles);
     if (c->precision == SRBE_MIXED)
-      k_sfac_partial<true><<<grid, kSfThreads, 0, c->stream>>>(n, x, y, z, u, w, w32, K, c->dm.p, invL, c->tab.p,
+      k_sfac_partial<true><<<grid, kSfThreads, 0, c->stream>>>(n, x, y, z, u, w, w32, K, c->dm.p, invL, c->tabi.p,
                                                                chunk, c->partial.p, c->mpart.p, f, c->sfdone.p);
     else
       k_sfac_partial<false><<<grid, kSfThreads, 0, c->stream>>>(n, x, y, z, u, w, nullptr, K, c->dm.p, invL,
-                                                                c->tab.p, chunk, c->partial.p, c->mpart.p, f,
+                                                                c->tabi.p, chunk, c->partial.p, c->mpart.p, f,
                                                                 c->sfdone.p);
     c->launches++;
     c->mode_evals += n * (int64_t)K;

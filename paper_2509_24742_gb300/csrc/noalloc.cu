@@ -24,12 +24,12 @@ constexpr int kNaMaxChunks = 1024;
 constexpr int kNaMaxDevices = 64;
 
 static __device__ __align__(256) double2 na_scratch[kNaPartials];
-static __device__ __align__(256) double2 na_table[kTab];
+static __device__ __align__(256) longlong2 na_table[kTab];
 
 struct DeviceSetup {
   bool ready = false;
   double2 *scratch = nullptr;
-  double2 *table = nullptr;
+  longlong2 *table = nullptr;
 };
 DeviceSetup g_setup[kNaMaxDevices];
 std::mutex g_setup_mutex;
@@ -37,7 +37,7 @@ std::mutex g_setup_mutex;
 // partial[c][k] = sum over particles of chunk c of w_j exp(i k . r_j); r is [n][3], m is [K][3]
 __global__ void __launch_bounds__(kNaThreads)
 k_na_partial(int64_t n, const double *__restrict__ r, const double *__restrict__ w, int K,
-             const int32_t *__restrict__ m3, double3 invL, const double2 *__restrict__ tab, int64_t chunk,
+             const int32_t *__restrict__ m3, double3 invL, const longlong2 *__restrict__ tab, int64_t chunk,
              double2 *__restrict__ partial) {
   __shared__ uint64_t su[3][kNaThreads];
   __shared__ double sw[kNaThreads];
@@ -111,11 +111,8 @@ int setup_device(DeviceSetup **out) {
   if (!s.ready) {
     if (cudaGetSymbolAddress((void **)&s.scratch, na_scratch) != cudaSuccess) return SRBE_ECUDA;
     if (cudaGetSymbolAddress((void **)&s.table, na_table) != cudaSuccess) return SRBE_ECUDA;
-    double2 h[kTab];
-    for (int j = 0; j < kTab; ++j) {
-      const long double a = 2.0L * 3.141592653589793238462643383279502884L * (long double)j / (long double)kTab;
-      h[j] = make_double2((double)cosl(a), (double)sinl(a));
-    }
+    longlong2 h[kTab];
+    fix_table(h);
     if (cudaMemcpyToSymbol(na_table, h, sizeof(h)) != cudaSuccess) return SRBE_ECUDA;
     // A copy from pageable memory may return before its DMA has landed, and streams created
     // non-blocking do not wait for the legacy stream it ran on: wait for it here, so that a first

@@ -557,8 +557,8 @@ __device__ __forceinline__ void pair_ion_ele(const PairSite &S, const CellsDev &
 
 // The FP64 form's pair sums (pairfix.cuh): coordinates as fractions of the period W, radial factors from
 // tables in r^2.  Measured on GB300 against the plain FP64 functions (sqrt, erfc, exp, divisions), whole
-// force kernel: 8,000 + 3,072 sites 1,279 -> 267 us, 45,692 + 6,144 sites 12.8 -> 2.34 ms; the rms error of a
-// pair's force against 64 bits is the same or smaller (checked term by term against long double arithmetic).
+// force kernel: 8,000 + 3,072 sites 1,279 -> 195 us, 45,692 + 6,144 sites 12.8 -> 1.68 ms; the rms error of a
+// pair's force against 64 bits is smaller (checked term by term against long double arithmetic).
 struct PairFix {
   uint64_t Lx, Ly;              // the box edges as fractions of W
   uint64_t rc2;                 // rc^2 as S
@@ -578,9 +578,10 @@ __device__ __forceinline__ void pair_add(const PairFix &fx, double fs, int64_t d
   f[1] = fma(fs, fix_to_double(dy, fx.e), f[1]);
   f[2] = fma(fs, fix_to_double(dz, fx.e), f[2]);
 }
-__device__ __forceinline__ double pair_lj(double2 ab, const PairArg &p, uint64_t Sv) {
-  const double u = pair_recip(p.s, pair_s_float(Sv)), u2 = u * u;
-  return fma(ab.x, u2 * u, -ab.y) * (u2 * u2);
+__device__ __forceinline__ double pair_lj(double2 ab, const PairArg &p) {
+  double u3, u4;
+  pair_powers(p, u3, u4);
+  return fma(ab.x, u3, -ab.y) * u4;
 }
 
 __device__ __forceinline__ void pair_ion_ion_fix(const PairSite &S, const CellsDev &ions, const MdDev &md,
@@ -595,7 +596,7 @@ __device__ __forceinline__ void pair_ion_ion_fix(const PairSite &S, const CellsD
   }
   const PairArg p = pair_arg(Sv);
   double lj = 0.0;
-  if (md.ntype && ions.ms[e.x] != S.mi) lj = pair_lj(md.ljp[S.ti * md.ntype + ions.ts[e.x]], p, Sv);
+  if (md.ntype && ions.ms[e.x] != S.mi) lj = pair_lj(md.ljp[S.ti * md.ntype + ions.ts[e.x]], p);
   const double fs = fma(S.qi * ions.ws[e.x], pair_poly(fx.ii[p.idx], p), lj);
   pair_add(fx, fs, dx, dy, dz, A.l);
 }
@@ -611,7 +612,7 @@ __device__ __forceinline__ void pair_ion_ele_fix(const PairSite &S, const CellsD
     return;
   }
   const PairArg p = pair_arg(Sv);
-  const double lj = md.ntype ? pair_lj(md.ljp[S.ti * md.ntype + (md.ntype - 1)], p, Sv) : 0.0;
+  const double lj = md.ntype ? pair_lj(md.ljp[S.ti * md.ntype + (md.ntype - 1)], p) : 0.0;
   const double fs = fma(S.qi * Q[eles.order[e.x]], pair_poly(fx.ie[p.idx], p), lj);
   pair_add(fx, fs, dx, dy, dz, A.l);
 }
@@ -865,7 +866,7 @@ __global__ void __launch_bounds__(kGatherThreads)
 k_electrode_rhs(int64_t ne, const double *__restrict__ ex, const double *__restrict__ ey,
                 const double *__restrict__ ez, const uint64_t *__restrict__ eu, int K, const int4 *__restrict__ modes,
                 const double2 *__restrict__ coefS, const float2 *__restrict__ coefS32,
-                const double2 *__restrict__ tab, double3 invL, CellsDev ions, ListsDev nl,
+                const longlong2 *__restrict__ tab, double3 invL, CellsDev ions, ListsDev nl,
                 double Lx, double Ly, double alpha, double eta, double rc, double slab, const double *__restrict__ scal,
                 double *__restrict__ b, float2 *__restrict__ bsplit, const double *__restrict__ bfar,
                 const float4 *__restrict__ epf, ForceF32 pf, const uint64_t *__restrict__ euw, PairFix fx) {
@@ -1438,13 +1439,13 @@ void electrode_rhs(srbe_ctx *c) {
   if (c->precision == SRBE_MIXED)
     k_electrode_rhs<true><<<nb, kGatherThreads, 0, c->stream>>>(c->ne, c->ex.p, c->ey.p, c->ez.p, c->eu.p, K, c->dm.p,
                                                                coef,
-                                                               c->coef32.p, c->tab.p, invL, ions, lists_dev(c), c->L[0], c->L[1], c->alpha,
+                                                               c->coef32.p, c->tabi.p, invL, ions, lists_dev(c), c->L[0], c->L[1], c->alpha,
                                                                c->eta, c->rc, slab, c->scal.p, c->bvec.p, c->bsplit.p,
                                                                bfar, c->epf.p, pf, c->euw.p, pair_fix(c));
   else
     k_electrode_rhs<false><<<nb, kGatherThreads, 0, c->stream>>>(c->ne, c->ex.p, c->ey.p, c->ez.p, c->eu.p, K, c->dm.p,
                                                                coef,
-                                                                c->coef32.p, c->tab.p, invL, ions, lists_dev(c), c->L[0], c->L[1], c->alpha,
+                                                                c->coef32.p, c->tabi.p, invL, ions, lists_dev(c), c->L[0], c->L[1], c->alpha,
                                                                 c->eta, c->rc, slab, c->scal.p, c->bvec.p, c->bsplit.p,
                                                                 bfar, c->epf.p, pf, c->euw.p, pair_fix(c));
   c->launches++;
@@ -1478,7 +1479,7 @@ __global__ void __launch_bounds__(kGatherThreads)
 k_ion_forces(int64_t ni, CellsDev ions, CellsDev eles, ListsDev nl, const double *__restrict__ Q,
              const float *__restrict__ Q32,
              int K, const int4 *__restrict__ modes, const double2 *__restrict__ coefF,
-             const float2 *__restrict__ coefF32, const double2 *__restrict__ tab,
+             const float2 *__restrict__ coefF32, const longlong2 *__restrict__ tab,
              double3 invL, float3 kvf, double Lx, double Ly, double alpha, double eta, double rc, double slab,
              ForceF32 pf, const double *__restrict__ scal, MdDev md, const double *__restrict__ x_orig,
              const double *__restrict__ y_orig, const double *__restrict__ z_orig, double *__restrict__ F,
@@ -1964,7 +1965,7 @@ void ion_forces(srbe_ctx *c, bool energies) {
     const ForceF32 pf{(float)c->L[0], (float)c->L[1], (float)c->alpha, (float)c->eta,
                       (float)c->rc,   (float)slab,   (float)md.kb};
     kern<<<nblk, kGatherThreads, 0, c->stream>>>(c->ni, ions, eles, lists_dev(c), c->Q.p, c->Q32.p, K, c->dm.p, coef,
-                                                 c->coef32.p, c->tab.p, invL, kvf, c->L[0], c->L[1], c->alpha, c->eta,
+                                                 c->coef32.p, c->tabi.p, invL, kvf, c->L[0], c->L[1], c->alpha, c->eta,
                                                  c->rc, slab, pf, c->scal.p, md, c->x.p, c->y.p, c->z.p, c->F.p, ep,
                                                  part2 ? c->fii.p : nullptr, pair_fix(c), c->kv.p);
     c->launches++;

@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdio>
 #include <string>
 #include <vector>
@@ -260,6 +261,7 @@ struct srbe_ctx {
   srbe::DevBuf<double> dc;
   srbe::DevBuf<double2> S1, S2;                // structure factors (S2 holds S1 + S2 after the update)
   srbe::DevBuf<double2> tab;                   // sin/cos table
+  srbe::DevBuf<longlong2> tabi;                // the same in Q62 (FP64 form's per-step sums)
 
   // pinned staging for mode lists
   int4 *h_mode_stage = nullptr;
@@ -394,20 +396,21 @@ __device__ __forceinline__ void sincos_turns(uint64_t th, const double2 *__restr
   s = fma(T.y, cm1, fma(T.x, sx, T.y));
 }
 
-// The same in the FP64 form's per-step sums (structure factors, b, force gather): the remainder x gives
-// cos x - 1 and sin x in integer arithmetic (fixphase.cuh), which leaves the four FP64 multiply-adds of the
-// angle addition; the function above needs twelve FP64 operations, 7 clocks of an SM.  The rms error is
-// 4.66e-17 either way (table and roundings).  The set-up of A and the lattice phases, a few evaluations
-// per step at most, keep the function above and so A's bits.
-__device__ __forceinline__ void sincos_turns_fix(uint64_t th, const double2 *__restrict__ tab, double &c, double &s) {
-  const uint64_t t = th + (1ull << 53);
-  const unsigned idx = (unsigned)(t >> 54);
-  const int64_t rem = (int64_t)(th - ((uint64_t)idx << 54));     // in [-2^53, 2^53)
-  double cm1, sx;
-  small_cos_sin(rem, cm1, sx);
-  const double2 T = __ldg(&tab[idx]);
-  c = fma(T.x, cm1, fma(-T.y, sx, T.x));
-  s = fma(T.y, cm1, fma(T.x, sx, T.y));
+// The same in the FP64 form's per-step sums (structure factors, b, force gather), in integer arithmetic
+// (fixphase.cuh): the function above needs twelve FP64 operations, 7 clocks of an SM.  rms error 4.66e-17
+// there, 2.71e-17 here.  The set-up of A and the lattice phases, a few evaluations per step at most, keep the
+// function above and so A's bits.
+__device__ __forceinline__ void sincos_turns_fix(uint64_t th, const longlong2 *__restrict__ tab, double &c, double &s) {
+  phase_cos_sin(th, __ldg(&tab[phase_index(th)]), c, s);
+}
+
+// host: the table of sincos_turns_fix, kTab entries
+inline void fix_table(longlong2 *h) {
+  for (int j = 0; j < kTab; ++j) {
+    const long double a = 2.0L * 3.141592653589793238462643383279502884L * (long double)j / (long double)kTab;
+    h[j].x = (long long)llroundl(cosl(a) * 4611686018427387904.0L);
+    h[j].y = (long long)llroundl(sinl(a) * 4611686018427387904.0L);
+  }
 }
 
 // mode k's integer vector as doubles (SoA), so that the gather over ions needs no conversions
