@@ -557,7 +557,7 @@ __device__ __forceinline__ void pair_ion_ele(const PairSite &S, const CellsDev &
 
 // The FP64 form's pair sums (pairfix.cuh): coordinates as fractions of the period W, radial factors from
 // tables in r^2.  Measured on GB300 against the plain FP64 functions (sqrt, erfc, exp, divisions), whole
-// force kernel: 8,000 + 3,072 sites 1,279 -> 195 us, 45,692 + 6,144 sites 12.8 -> 1.68 ms; the rms error of a
+// force kernel: 8,000 + 3,072 sites 1,279 -> 145 us, 45,692 + 6,144 sites 12.8 -> 1.28 ms; the rms error of a
 // pair's force against 64 bits is smaller (checked term by term against long double arithmetic).
 struct PairFix {
   uint64_t Lx, Ly;              // the box edges as fractions of W
@@ -584,20 +584,42 @@ __device__ __forceinline__ double pair_lj(double2 ab, const PairArg &p) {
   return fma(ab.x, u3, -ab.y) * u4;
 }
 
+// Pairs closer than the tables reach: the plain functions, in calls of their own (one in a few million
+// pairs; inlined, their registers and code weigh on every other).
+__device__ __noinline__ double pair_near_force(double r2, double alpha, double eta, double qq, double2 sg) {
+  double phi, md2;
+  if (eta > 0.0) pair_ie(r2, alpha, eta, phi, md2);
+  else pair_ii(r2, alpha, phi, md2);
+  const double sr2 = sg.x / r2, sr6 = sr2 * sr2 * sr2;
+  return fma(kKe, qq * md2, 24.0 * sg.y * (2.0 * sr6 * sr6 - sr6) / r2);
+}
+__device__ __noinline__ double pair_near_phi(double r2, double alpha, double eta) {
+  double phi, md2;
+  pair_ie(r2, alpha, eta, phi, md2);
+  return phi;
+}
+__device__ __forceinline__ double pair_r2(const PairFix &fx, int64_t dx, int64_t dy, int64_t dz) {
+  const double x = fix_to_double(dx, fx.e), y = fix_to_double(dy, fx.e), z = fix_to_double(dz, fx.e);
+  return x * x + y * y + z * z;
+}
+
 __device__ __forceinline__ void pair_ion_ion_fix(const PairSite &S, const CellsDev &ions, const MdDev &md,
                                                  const PairFix &fx, int2 e, PairAcc &A) {
   int64_t dx, dy, dz;
   pair_diff(S, fx, ions.uw, ions.n, e, dx, dy, dz);
   const uint64_t Sv = pair_S(dx, dy, dz);
   if (Sv >= fx.rc2) return;
-  if (Sv < kPtMin) {            // closer than the tables reach
-    pair_ion_ion<false, false>(S, ions, md, e, A);
-    return;
+  const double qq = S.qi * ions.ws[e.x];
+  const bool with_lj = md.ntype && ions.ms[e.x] != S.mi;
+  double fs;
+  if (Sv < kPtMin) {
+    const double2 sg = with_lj ? md.lj[S.ti * md.ntype + ions.ts[e.x]] : make_double2(0.0, 0.0);
+    fs = pair_near_force(pair_r2(fx, dx, dy, dz), S.alpha, 0.0, qq, sg);
+  } else {
+    const PairArg p = pair_arg(Sv);
+    const double lj = with_lj ? pair_lj(md.ljp[S.ti * md.ntype + ions.ts[e.x]], p) : 0.0;
+    fs = fma(qq, pair_poly(fx.ii[p.idx], p), lj);
   }
-  const PairArg p = pair_arg(Sv);
-  double lj = 0.0;
-  if (md.ntype && ions.ms[e.x] != S.mi) lj = pair_lj(md.ljp[S.ti * md.ntype + ions.ts[e.x]], p);
-  const double fs = fma(S.qi * ions.ws[e.x], pair_poly(fx.ii[p.idx], p), lj);
   pair_add(fx, fs, dx, dy, dz, A.l);
 }
 
@@ -606,14 +628,17 @@ __device__ __forceinline__ void pair_ion_ele_fix(const PairSite &S, const CellsD
   int64_t dx, dy, dz;
   pair_diff(S, fx, eles.uw, eles.n, e, dx, dy, dz);
   const uint64_t Sv = pair_S(dx, dy, dz);
-  if (Sv >= fx.rc2) return;
+  if (Sv >= fx.rc2 || Sv == 0) return;
+  const double qq = S.qi * Q[eles.order[e.x]];
+  double fs;
   if (Sv < kPtMin) {
-    pair_ion_ele<false, false>(S, eles, md, Q, nullptr, e, A);
-    return;
+    const double2 sg = md.ntype ? md.lj[S.ti * md.ntype + (md.ntype - 1)] : make_double2(0.0, 0.0);
+    fs = pair_near_force(pair_r2(fx, dx, dy, dz), S.alpha, S.eta, qq, sg);
+  } else {
+    const PairArg p = pair_arg(Sv);
+    const double lj = md.ntype ? pair_lj(md.ljp[S.ti * md.ntype + (md.ntype - 1)], p) : 0.0;
+    fs = fma(qq, pair_poly(fx.ie[p.idx], p), lj);
   }
-  const PairArg p = pair_arg(Sv);
-  const double lj = md.ntype ? pair_lj(md.ljp[S.ti * md.ntype + (md.ntype - 1)], p) : 0.0;
-  const double fs = fma(S.qi * Q[eles.order[e.x]], pair_poly(fx.ie[p.idx], p), lj);
   pair_add(fx, fs, dx, dy, dz, A.l);
 }
 
@@ -703,7 +728,9 @@ __device__ __forceinline__ void compacted_list(const PairSite &S, const CellsDev
                                                int count, float cut2, int2 *q, int lane, Pair &&pair) {
   int qn = 0;
   const unsigned below = (1u << lane) - 1u;
-  for (int base = 0; base < count; base += 32) {
+  // one call site for the full batches and the rest: the pair's code is long, and a second copy of it in
+  // each of the force kernel's two lists costs instruction fetches
+  for (int base = 0; base < count || qn > 0; base += 32) {
     const int k = base + lane;
     bool in = false;
     int pp = 0, img = 0;
@@ -720,18 +747,15 @@ __device__ __forceinline__ void compacted_list(const PairSite &S, const CellsDev
     const unsigned m = __ballot_sync(0xffffffffu, in);
     if (in) q[qn + __popc(m & below)] = make_int2(pp, img);
     qn += __popc(m);
-    if (qn >= 32) {
+    if (qn >= 32 || base + 32 >= count) {
       __syncwarp();
-      pair(q[lane]);
+      if (lane < qn) pair(q[lane]);
       __syncwarp();
       if (lane < qn - 32) q[lane] = q[lane + 32];
       __syncwarp();
-      qn -= 32;
+      qn = max(qn - 32, 0);
     }
   }
-  __syncwarp();
-  if (lane < qn) pair(q[lane]);
-  __syncwarp();
 }
 
 // FP32 passes over one Verlet list (the mixed form's forces): 32 entries per batch with a
@@ -938,11 +962,8 @@ k_electrode_rhs(int64_t ne, const double *__restrict__ ex, const double *__restr
         const PairArg p = pair_arg(Sv);
         phi = pair_poly(fx.phi[p.idx], p);
       } else {                  // closer than the tables reach
-        const double ddx = X - (ions.xs[pp] + ix * Lx), ddy = Y - (ions.ys[pp] + iy * Ly), ddz = Z - ions.zs[pp];
-        const double r2 = ddx * ddx + ddy * ddy + ddz * ddz;
-        double md;
-        if (r2 == 0.0) return;
-        pair_ie(r2, alpha, eta, phi, md);
+        if (Sv == 0) return;
+        phi = pair_near_phi(pair_r2(fx, dx, dy, dz), alpha, eta);
       }
       near = fma(-ions.ws[pp], phi, near);
     }
@@ -1474,8 +1495,11 @@ __device__ __forceinline__ double widen_f32(float f) {
 // PART 0: the whole force.  PART 2 (mixed form without energies): everything but the ion-ion pairs
 // and bonds, plus Fii, their forces from k_ion_ii (sorted order; they need neither Q nor S, so that
 // pass runs beside b, the solve and S2)
+// The FP64 form's pair sums are long dependent chains of integer instructions (18 warps of an SM issue 1.6
+// instructions per clock): 64 registers and 32 warps, with a few spills, measured best at 8,000 + 3,072 sites:
+// 195 us with 106 registers, 178 with 80, 145 with 64; 48 registers gain nothing more.
 template <bool F32, bool EN, int PART>
-__global__ void __launch_bounds__(kGatherThreads)
+__global__ void __launch_bounds__(kGatherThreads, F32 || EN ? 1 : 4)
 k_ion_forces(int64_t ni, CellsDev ions, CellsDev eles, ListsDev nl, const double *__restrict__ Q,
              const float *__restrict__ Q32,
              int K, const int4 *__restrict__ modes, const double2 *__restrict__ coefF,
@@ -1514,6 +1538,9 @@ k_ion_forces(int64_t ni, CellsDev ions, CellsDev eles, ListsDev nl, const double
     const uint64_t ux = ions.us[p], uy = ions.us[ni + p], uz = ions.us[2 * ni + p];
     const double tpx = 2.0 * kPi * invL.x, tpy = 2.0 * kPi * invL.y, tpz = 2.0 * kPi * invL.z;
     // ---- k-space gather
+    // the FP64 form without energies takes the fixed-point pair sums
+    constexpr bool kFix = !F32 && !EN;
+    PairAcc A;
     double fk[3] = {0, 0, 0};
     float ak0 = 0.f, ak1 = 0.f, ak2 = 0.f;
     if (!F32) {
@@ -1530,6 +1557,10 @@ k_ion_forces(int64_t ni, CellsDev ions, CellsDev eles, ListsDev nl, const double
       fk[0] *= tpx;
       fk[1] *= tpy;
       fk[2] *= tpz;
+      if (kFix) {               // in kJ/mol/nm from here on, in the pairs' accumulators
+#pragma unroll
+        for (int d = 0; d < 3; ++d) A.l[d] = -kKe * qi * fk[d];
+      }
     } else {
       const uint32_t vx = (uint32_t)(ux >> 32), vy = (uint32_t)(uy >> 32), vz = (uint32_t)(uz >> 32);
       for (int k = lane; k < K; k += 32) {
@@ -1551,14 +1582,11 @@ k_ion_forces(int64_t ni, CellsDev ions, CellsDev eles, ListsDev nl, const double
     S.Lxf = pf.Lx; S.Lyf = pf.Ly; S.af = pf.alpha; S.etaf = pf.eta;
     S.qke = (float)kKe * self.w;
     S.ti = ti; S.mi = mi; S.p = p;
-    // the FP64 form without energies takes the fixed-point pair sums
-    constexpr bool kFix = !F32 && !EN;
     if (kFix) {
       S.ux = ions.uw[p]; S.uy = ions.uw[ni + p]; S.uz = ions.uw[2 * ni + p];
     }
     const float rcf = F32 ? pf.rc : (float)rc;
     const float cut2 = F32 ? rcf * rcf : (rcf + kPrecheckMargin) * (rcf + kPrecheckMargin);
-    PairAcc A;
     int2 *q = wq[warp];
     auto ion_pair = [&](int2 e) {
       if constexpr (kFix) pair_ion_ion_fix(S, ions, md, fx, e, A);
@@ -1638,10 +1666,7 @@ k_ion_forces(int64_t ni, CellsDev ions, CellsDev eles, ListsDev nl, const double
       }
     } else if (kFix) {
       // everything in kJ/mol/nm per lane, then one sum over the warp; lanes 0, 8 and 16 finish x, y, z
-      double v[3];
-#pragma unroll
-      for (int d = 0; d < 3; ++d) v[d] = fma(kKe, fma(-qi, fk[d], rr[d]), ll[d]);
-      double f = warp_sum3(v[0], v[1], v[2], lane);
+      double f = warp_sum3(ll[0], ll[1], ll[2], lane);
       if (lane == 0 || lane == 8 || lane == 16) {
         const int d = lane >> 3;
         // slab force: M_z = sum q_i z_i + sum Q_j Z_j
