@@ -874,7 +874,9 @@ __device__ float block_rows_cached(const PcgArgs &a, const float4 *sA, const flo
   for (int t = 0; t < kCacheVecs; ++t) {
     const int j = c0 + lane + 32 * t;
     uv[t] = j < c1 ? __ldcg(reinterpret_cast<const float4 *>(u) + j) : zero;
-    col[t] = j < c1 ? j : c0;                // a valid column; its u is zero
+    // without a column of its own the lane reads column 0 (its u is zero): c0 itself lies past the row
+    // where 7 seg >= nv, the last warps of electrodes of up to 196 sites
+    col[t] = j < c1 ? j : 0;
   }
   auto fetch = [&](int r0) {
 #pragma unroll

@@ -28,3 +28,25 @@ def test_mixed_pcg_reaches_the_direct_charges(nx, ny):
     assert 0 < it < 5000 and res <= tol and res64 <= 10 * tol
     assert np.linalg.norm(Q1 - Q0) <= 1e3 * tol * np.linalg.norm(Q0)
     assert abs(psi1 - psi0) <= 1e3 * tol * abs(psi0)
+
+
+@pytest.mark.parametrize("nx,ny,gone", [(3, 2, 0), (4, 3, 0), (17, 1, 2), (6, 3, 0), (7, 4, 0), (11, 3, 2)])
+def test_mixed_pcg_on_small_electrodes(nx, ny, gone):
+    """36, 72, 100, 108, 168 and 196 sites: the last of a block's eight column segments of the cached product
+    start at or past the end of the row (100 and 196 also have blocks with fewer rows than others).  The
+    bounds above: the sites are at least as far apart."""
+    tol = 1e-8
+    s = wl.make_slab("pcg", (max(1.5, 0.25 * nx), 1.5, 12.0), nx, ny, 40, 1, alpha=3.5, eta_inv=19.79, rc=1.0, P=30,
+                     M=2, seed=7)
+    keep = np.arange(gone, s.R.shape[0])
+    s.R, s.side = s.R[keep], s.side[keep]
+    with srbe.from_slab(s, precision=srbe.MIXED) as ctx:
+        ctx.sample_k(3, 0)
+        Q0, psi0, _ = ctx.solve_charges()
+        ctx.set_solver(srbe.PCG, tol=tol, maxit=5000, warm=srbe.WARM_ZERO)
+        for _ in range(3):
+            Q1, psi1, _ = ctx.solve_charges()
+            it, res = ctx.solver_stats()
+            assert 0 < it < 5000 and res <= tol and ctx.charge_residual() <= 10 * tol
+            assert np.linalg.norm(Q1 - Q0) <= 1e3 * tol * np.linalg.norm(Q0)
+            assert abs(psi1 - psi0) <= 1e3 * tol * abs(psi0)
