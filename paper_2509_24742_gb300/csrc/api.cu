@@ -2026,7 +2026,6 @@ int srbe_get_solver_stats(srbe_ctx *c, int *iterations, double *rel_residual) {
 namespace {
 void mlp_alloc(srbe_ctx *c) {
   const size_t n = (size_t)mlp_param_count();
-  c->mlp.split_ready = false;
   c->mlp.P.ensure(n);
   c->mlp.m1.ensure(n);
   c->mlp.m2.ensure(n);
@@ -2066,6 +2065,7 @@ int srbe_mlp_init(srbe_ctx *c, uint64_t seed) {
     P[o++] = 1.f;                               // target spread
     mlp_alloc(c);
     SRBE_CUDA(cudaMemcpyAsync(c->mlp.P.p, P.data(), sizeof(float) * n, cudaMemcpyHostToDevice, c->stream));
+    mlp_split(c);
     mlp_reset_moments(c);
     SRBE_CUDA(cudaStreamSynchronize(c->stream));
     c->mlp.ready = true;
@@ -2089,6 +2089,7 @@ int srbe_mlp_set_params(srbe_ctx *c, const float *params, int64_t count) {
     for (int64_t i = 0; i < count; ++i) SRBE_REQUIRE(std::isfinite(params[i]), SRBE_EINVAL, "non-finite parameter");
     mlp_alloc(c);
     SRBE_CUDA(cudaMemcpyAsync(c->mlp.P.p, params, sizeof(float) * count, cudaMemcpyHostToDevice, c->stream));
+    mlp_split(c);
     mlp_reset_moments(c);
     SRBE_CUDA(cudaStreamSynchronize(c->stream));
     c->mlp.ready = true;
@@ -2232,7 +2233,6 @@ int srbe_mlp_train(srbe_ctx *c, const float *D, const float *target, int64_t n, 
     P[oYm] = (float)m;
     P[oYs] = (float)std::max(std::sqrt(std::max(ts2 / n - m * m, 0.0)), 1e-12);
     SRBE_CUDA(cudaMemcpyAsync(c->mlp.P.p, P.data(), sizeof(float) * np, cudaMemcpyHostToDevice, c->stream));
-    c->mlp.split_ready = false;
     double last = 0.0;
     for (int e = 0; e < epochs; ++e) {
       shuffle.wait();
@@ -2244,6 +2244,7 @@ int srbe_mlp_train(srbe_ctx *c, const float *D, const float *target, int64_t n, 
         mlp_grad_step(c, c->mlp.data_D.p, c->mlp.data_T.p, c->mlp.rows.p + b0, nb, nullptr, true, lr, weight_decay,
                       dl + k);
       }
+      if (e + 1 == epochs) mlp_split(c);
       SRBE_CUDA(cudaMemcpyAsync(err2.data(), dl, sizeof(double) * nbatch, cudaMemcpyDeviceToHost, c->stream));
       SRBE_CUDA(cudaStreamSynchronize(c->stream));
       double tot = 0.0;

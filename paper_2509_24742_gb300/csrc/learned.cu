@@ -681,6 +681,16 @@ void mlp_descriptors(srbe_ctx *c, float *D_dev) {
   SRBE_CUDA(cudaGetLastError());
 }
 
+// The forward pass's operands from the parameters: queued by every call that changes them, not by the pass
+// itself, so that a prediction captured in a CUDA graph (by a caller, or in a captured step) holds no split
+// of its own, allocates nothing and reads the parameters as they are when it is replayed.
+void mlp_split(srbe_ctx *c) {
+  k_mlp_split<<<blocks_for(kH * kH, 256), 256, 0, c->stream>>>(
+      c->mlp.P.p, reinterpret_cast<__nv_bfloat16 *>(c->mlp.split.ensure(kTcWeights)));
+  c->launches++;
+  SRBE_CUDA(cudaGetLastError());
+}
+
 void mlp_forward(srbe_ctx *c, const float *D_dev, int64_t n, float *out_dev, double *out_y_dev) {
   if (n <= 0) return;
   static int nsm = 0;
@@ -690,12 +700,7 @@ void mlp_forward(srbe_ctx *c, const float *D_dev, int64_t n, float *out_dev, dou
     SRBE_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     SRBE_CUDA(cudaFuncSetAttribute(k_mlp_forward_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmem));
   }
-  __nv_bfloat16 *W = reinterpret_cast<__nv_bfloat16 *>(c->mlp.split.ensure(kTcWeights));
-  if (!c->mlp.split_ready) {
-    k_mlp_split<<<blocks_for(kH * kH, 256), 256, 0, c->stream>>>(c->mlp.P.p, W);
-    c->launches++;
-    c->mlp.split_ready = true;
-  }
+  const __nv_bfloat16 *W = reinterpret_cast<const __nv_bfloat16 *>(c->mlp.split.p);
   const unsigned grid = (unsigned)std::min<int64_t>((n + 127) / 128, nsm);
   k_mlp_forward_tc<<<grid, kTcThreads, kTcSmem, c->stream>>>(n, D_dev, c->mlp.P.p, W, out_dev, out_y_dev,
                                                              c->d_status);
@@ -734,10 +739,7 @@ void mlp_grad_step(srbe_ctx *c, const float *D_dev, const float *T_dev, const in
     m.gpart.ensure((size_t)nslot * kNtrain);
     m.lpart.ensure((size_t)nslot);
   }
-  if (apply) {
-    m.t++;
-    m.split_ready = false;
-  }
+  if (apply) m.t++;
   const AdamW opt{m.P.p, m.m1.p, m.m2.p, m.t, lr, wd};
   for (int64_t b0 = 0; b0 < n; b0 += kTrChunk) {
     const int64_t nb = std::min(kTrChunk, n - b0);

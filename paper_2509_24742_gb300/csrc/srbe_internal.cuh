@@ -126,8 +126,7 @@ struct MlpState {
   bool ready = false;
   int t = 0;
   DevBuf<float> P, m1, m2, gpart, grad, D, data_D, data_T;
-  DevBuf<uint16_t> split;            // W1, W2 as blocked BF16 (hi, lo) operands of the forward pass
-  bool split_ready = false;          // false once the parameters have changed
+  DevBuf<uint16_t> split;            // W1, W2 as blocked BF16 (hi, lo) operands of the forward pass (mlp_split)
   DevBuf<float> act;                 // activations of a training pass, row-major
   DevBuf<double> lpart, loss;        // squared errors: per split, per minibatch of an epoch
   DevBuf<double2> Slow;
@@ -462,6 +461,7 @@ void pcg_prepare(srbe_ctx *c);
 int mlp_param_count();
 int mlp_input_width();
 void mlp_descriptors(srbe_ctx *c, float *D_dev);
+void mlp_split(srbe_ctx *c);
 void mlp_forward(srbe_ctx *c, const float *D_dev, int64_t n, float *out_dev, double *out_y_dev);
 void mlp_grad_step(srbe_ctx *c, const float *D_dev, const float *T_dev, const int32_t *rows_dev, int64_t n,
                    float *grad_dev, bool apply, float lr, float wd, double *loss_dev);
