@@ -693,13 +693,10 @@ void mlp_split(srbe_ctx *c) {
 
 void mlp_forward(srbe_ctx *c, const float *D_dev, int64_t n, float *out_dev, double *out_y_dev) {
   if (n <= 0) return;
-  static int nsm = 0;
-  if (!nsm) {
-    int dev = 0;
-    SRBE_CUDA(cudaGetDevice(&dev));
-    SRBE_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  static KernelSetup setup;
+  const int nsm = setup.sms([] {
     SRBE_CUDA(cudaFuncSetAttribute(k_mlp_forward_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmem));
-  }
+  });
   const __nv_bfloat16 *W = reinterpret_cast<const __nv_bfloat16 *>(c->mlp.split.p);
   const unsigned grid = (unsigned)std::min<int64_t>((n + 127) / 128, nsm);
   k_mlp_forward_tc<<<grid, kTcThreads, kTcSmem, c->stream>>>(n, D_dev, c->mlp.P.p, W, out_dev, out_y_dev,
@@ -713,17 +710,13 @@ void mlp_forward(srbe_ctx *c, const float *D_dev, int64_t n, float *out_dev, dou
 void mlp_grad_step(srbe_ctx *c, const float *D_dev, const float *T_dev, const int32_t *rows_dev, int64_t n,
                    float *grad_dev, bool apply, float lr, float wd, double *loss_dev) {
   auto &m = c->mlp;
-  static int nsm = 0;
   constexpr size_t kRowsSmem4 = sizeof(float) * (kH * (kW1s + kW2s) + 4 * (kIn + 3 * kH));
   constexpr size_t kRowsSmem8 = sizeof(float) * (kH * (kW1s + kW2s) + 8 * (kIn + 3 * kH));
-  if (!nsm) {
-    int dev = 0, v = 0;
-    SRBE_CUDA(cudaGetDevice(&dev));
-    SRBE_CUDA(cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev));
+  static KernelSetup setup;
+  const int nsm = setup.sms([] {
     SRBE_CUDA(cudaFuncSetAttribute(k_mlp_rows<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowsSmem4));
     SRBE_CUDA(cudaFuncSetAttribute(k_mlp_rows<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowsSmem8));
-    nsm = v;
-  }
+  });
   const int64_t nslot = (n + kTrSplit - 1) / kTrSplit, most = std::min(n, kTrChunk);
   const bool fused = nslot == 1;
   const int64_t rows_max = (most + 3) & ~(int64_t)3;     // keeps every array on a 16-byte boundary

@@ -8,6 +8,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -45,6 +46,26 @@ struct Error {
   do {                                                  \
     if (!(cond)) throw ::srbe::Error{(code), (text)};   \
   } while (0)
+
+// Settings of a kernel that hold per device (its shared-memory limit), made once for each device before any
+// thread launches it there; sms(fn) returns the device's number of SMs.  A setting that throws is made again
+// by the next call.
+struct KernelSetup {
+  static constexpr int kMax = 64;
+  std::once_flag once[kMax];
+  int nsm[kMax] = {};
+  template <class Fn>
+  int sms(Fn &&fn) {
+    int dev = 0;
+    SRBE_CUDA(cudaGetDevice(&dev));
+    SRBE_REQUIRE(dev >= 0 && dev < kMax, SRBE_ECUDA, "device index out of range");
+    std::call_once(once[dev], [&] {
+      SRBE_CUDA(cudaDeviceGetAttribute(&nsm[dev], cudaDevAttrMultiProcessorCount, dev));
+      fn();
+    });
+    return nsm[dev];
+  }
+};
 
 // ------------------------------------------------------------------------------------------------
 // device buffer with grow-only capacity

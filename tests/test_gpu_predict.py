@@ -1,15 +1,21 @@
-"""Prediction on device rows as part of a caller's own CUDA graph: a captured call (also a context's first
-prediction) is accepted, and a replay predicts with the parameters as they are by then, whether they were set,
-drawn anew or trained since.  Same kernel on the same operands: the same bits as an ordinary call."""
+"""The network's calls in a caller's own CUDA graph and from several threads.  Same kernels on the same operands
+as an ordinary call: the same bits."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
 from paper_2509_24742_gb300 import srbe
 
 pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 def test_captured_prediction_follows_the_parameters():
+    """A captured prediction (also a context's first one) is accepted, and a replay predicts with the parameters
+    as they are by then, whether they were set, drawn anew or trained since."""
     import torch
     rng = np.random.default_rng(2)
     D = torch.from_numpy(rng.gamma(2.0, 0.15, (333, srbe.N_DESC)).astype(np.float32)).cuda()
@@ -37,3 +43,37 @@ def test_captured_prediction_follows_the_parameters():
             assert np.array_equal(got, ref.cpu().numpy())
             assert all(not np.array_equal(got, s) for s in seen)
             seen.append(got)
+
+
+FIRST_CALLS = """
+import sys, threading, time
+import numpy as np
+from paper_2509_24742_gb300 import srbe
+train = sys.argv[1] == "train"
+ctxs = [srbe.Context((2.0, 2.0, 12.0), 3.5, 0.05, 1.2, 10, 2) for _ in range(12)]
+D = np.random.default_rng(0).gamma(2.0, 0.15, (700, srbe.N_DESC)).astype(np.float32)
+out, errors, start = [None] * len(ctxs), [], threading.Barrier(len(ctxs))
+for c in ctxs:
+    c.mlp_init(seed=1)
+def work(i):
+    try:
+        start.wait()
+        time.sleep(5e-5 * i)
+        out[i] = ctxs[i].mlp_gradients(D, D[:, 0])[0] if train else ctxs[i].mlp_predict(D)
+    except Exception as e:
+        errors.append(repr(e))
+threads = [threading.Thread(target=work, args=(i,)) for i in range(len(ctxs))]
+[t.start() for t in threads]
+[t.join() for t in threads]
+assert not errors, errors
+assert all(np.array_equal(o, out[0]) for o in out)
+"""
+
+
+@pytest.mark.parametrize("what", ["predict", "train"])
+def test_first_calls_of_several_threads(what):
+    """A process's first predictions (gradients), by twelve threads at once: none launches a kernel whose
+    shared-memory limit another thread is still setting."""
+    r = subprocess.run([sys.executable, "-c", FIRST_CALLS, what], cwd=ROOT, capture_output=True, text=True,
+                       timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
