@@ -836,7 +836,6 @@ __device__ float grid_gemv32_dot(const PcgArgs &a, const float *u, float *w) {
 // vector that is exchanged through memory.  What is left per iteration is two grid barriers, the load of
 // u and the reduction's partials, and 1 us of shared-memory reads.  3,072 sites: 8.9 us per iteration, 10.4 us
 // with rows streamed from L2 and the vectors in memory.
-constexpr int kPcgStaticSmem = 11264;      // bound of k_pcg_mixed's static shared memory
 constexpr int kCacheMaxN = 4096, kCacheVecs = kCacheMaxN / 4 / 8 / 32, kCacheMaxRows = 32;
 constexpr int kCacheGroup = 6, kCacheStream = 3;
 
@@ -1174,7 +1173,7 @@ void charge_update_pcg(srbe_ctx *c) {
     c->pcg.a32_ready = true;
   }
   // mixed form up to 4,096 sites: one block per SM, as many of its rows of A32 in shared memory as fit
-  // beside the kernel's own 11 KB (above, for n not a multiple of 4, and where the first warp's lanes are
+  // beside the kernel's own arrays (above, for n not a multiple of 4, and where the first warp's lanes are
   // fewer than a block's rows, every row streams from L2)
   const bool cache = mixed && n % 4 == 0 && n <= kCacheMaxN && (n + nsm - 1) / nsm <= kCacheMaxRows;
   const int most = cache ? nsm : blocks_per_sm * nsm;
@@ -1182,11 +1181,13 @@ void charge_update_pcg(srbe_ctx *c) {
   int srows = 0;
   if (cache) {
     int dev = 0, smem_max = 0;
+    cudaFuncAttributes fa;
     SRBE_CUDA(cudaGetDevice(&dev));
     SRBE_CUDA(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    SRBE_CUDA(cudaFuncSetAttribute(k_pcg_mixed, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   smem_max - kPcgStaticSmem));
-    srows = (int)std::min<int64_t>((n + grid - 1) / grid, (smem_max - kPcgStaticSmem) / (4 * n));
+    SRBE_CUDA(cudaFuncGetAttributes(&fa, k_pcg_mixed));
+    const int room = smem_max - (int)fa.sharedSizeBytes;
+    SRBE_CUDA(cudaFuncSetAttribute(k_pcg_mixed, cudaFuncAttributeMaxDynamicSharedMemorySize, room));
+    srows = (int)std::min<int64_t>((n + grid - 1) / grid, room / (4 * n));
   }
   const size_t smem = (size_t)srows * 4 * n;
   PcgArgs a;
