@@ -628,12 +628,14 @@ __device__ __forceinline__ void pair_ion_ele_fix(const PairSite &S, const CellsD
   int64_t dx, dy, dz;
   pair_diff(S, fx, eles.uw, eles.n, e, dx, dy, dz);
   const uint64_t Sv = pair_S(dx, dy, dz);
-  if (Sv >= fx.rc2 || Sv == 0) return;
+  if (Sv >= fx.rc2) return;
   const double qq = S.qi * Q[eles.order[e.x]];
   double fs;
   if (Sv < kPtMin) {
+    const double r2 = pair_r2(fx, dx, dy, dz);
+    if (r2 == 0.0) return;      // (S rounds to zero below 4e-10 R1 already)
     const double2 sg = md.ntype ? md.lj[S.ti * md.ntype + (md.ntype - 1)] : make_double2(0.0, 0.0);
-    fs = pair_near_force(pair_r2(fx, dx, dy, dz), S.alpha, S.eta, qq, sg);
+    fs = pair_near_force(r2, S.alpha, S.eta, qq, sg);
   } else {
     const PairArg p = pair_arg(Sv);
     const double lj = md.ntype ? pair_lj(md.ljp[S.ti * md.ntype + (md.ntype - 1)], p) : 0.0;
@@ -962,8 +964,9 @@ k_electrode_rhs(int64_t ne, const double *__restrict__ ex, const double *__restr
         const PairArg p = pair_arg(Sv);
         phi = pair_poly(fx.phi[p.idx], p);
       } else {                  // closer than the tables reach
-        if (Sv == 0) return;
-        phi = pair_near_phi(pair_r2(fx, dx, dy, dz), alpha, eta);
+        const double r2 = pair_r2(fx, dx, dy, dz);
+        if (r2 == 0.0) return;
+        phi = pair_near_phi(r2, alpha, eta);
       }
       near = fma(-ions.ws[pp], phi, near);
     }

@@ -54,3 +54,21 @@ def test_close_pairs_and_negative_z_match_oracle(orc):
     s.r[6] = [1.9999, 0.0001, 4.0]
     s.r[7] = [0.0002, 1.9998, 4.01]                    # across both periodic edges
     check(orc, s, False)
+
+
+@pytest.mark.parametrize("d", [1e-8, 2e-10, 1e-11])
+def test_ion_all_but_on_a_site(orc, d):
+    """An ion 1e-8 to 1e-11 nm above a site, where r^2 rounds to zero in the pair sums' units: it still raises that
+    site's potential (by -q 2 (1 / eta - alpha) / sqrt(pi), -19 q).  That term is (erfc(alpha r) - erfc(r / eta)) / r,
+    a difference of numbers next to one: a few 1.1e-16 / r of it are rounding, 1e-4 at 1e-11 nm, 5e-6 of the term.
+    The charges answer in proportion, so 1e-4 leaves a factor of 20."""
+    s = wl.make_slab("on", (2.0, 2.0, 12.0), 8, 8, 40, 1, alpha=3.0, eta_inv=19.79, rc=1.2, P=30, M=2, seed=4)
+    site = int(np.flatnonzero(s.R[:, 2] == 0.0)[9])
+    s.r[0] = s.R[site] + [0.0, 0.0, d]
+    samples = orc.sample_metropolis(s.box, s.alpha, s.M, s.P, 13, 0)
+    ref = orc.System(s, alpha_A=1.9)
+    ev = ref.evaluate(*ref.modes(samples), with_lj=False)
+    with srbe.from_slab(s, alpha_A=1.9) as ctx:
+        ctx.set_k(samples)
+        Q, _, _ = ctx.solve_charges()
+    assert np.linalg.norm(Q - ev["Q"]) < 1e-4 * np.linalg.norm(ev["Q"])
