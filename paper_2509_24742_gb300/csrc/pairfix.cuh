@@ -11,8 +11,8 @@
 //    exponent per interval, the tail in FP32 (its terms are below 2^-30 of 1 / r^3, the scale of a pair's
 //    force, so their FP32 rounding is below 2^-53 of it).  The error is bounded on that scale: 5e-16 of
 //    1 / r^3 at worst for any alpha r.  Of its own factor a screened pair has less: 2.4e-14 at worst, 2.9e-15 rms,
-//    at r = 1.2 nm with alpha 3.5 (plain functions 2.0e-15, 1.0e-15), 2.9e-12 at alpha r = 7, where the factor
-//    is 1e-20 of 1 / r^3;
+//    at r = 1.2 nm with alpha 3.5 (plain functions 2.0e-15, 1.0e-15), 2.9e-12 at alpha r = 7.2, where the factor
+//    is 3e-22 of 1 / r^3;
 //  * 1 / S comes from an FP32 reciprocal and one cubic Newton step, its powers from 64-bit products;
 //  * int64 <-> floating-point conversions are assembled with integer instructions.
 // A pair closer than R1 / 64 leaves the table and takes the plain FP64 functions.
