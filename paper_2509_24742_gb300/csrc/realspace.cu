@@ -11,6 +11,7 @@
 #include <cooperative_groups.h>
 
 #include "pairfix.cuh"
+#include "sfu.cuh"
 #include "srbe_internal.cuh"
 
 namespace cg = cooperative_groups;
@@ -278,24 +279,6 @@ __device__ __forceinline__ float erfc_as(float x, float ex2) {
   return poly * ex2;
 }
 
-// The special-function instructions without their handling of subnormal arguments and results (which no
-// pair within reach has): the same bits as rsqrtf, __expf and __fdividef(1, x) on normal numbers, about
-// eleven instructions per pair less.
-__device__ __forceinline__ float rsqrt_n(float x) {
-  float r;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-__device__ __forceinline__ float exp_n(float x) {
-  float r;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x * 1.4426950216293335f));
-  return r;
-}
-__device__ __forceinline__ float rcp_n(float x) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
 __device__ __forceinline__ float erfc_as_n(float x, float ex2) {
   const float t = rcp_n(fmaf(0.3275911f, x, 1.0f));
   const float poly = t * fmaf(t, fmaf(t, fmaf(t, fmaf(t, 1.061405429f, -1.453152027f), 1.421413741f),
