@@ -377,7 +377,8 @@ struct srbe::HostExt {
     double *hw = nullptr;
     const int4 *dhm = nullptr;    // the same buffers as device pointers
     const double *dhw = nullptr;
-    cudaGraphExec_t exec = nullptr;
+    cudaGraphExec_t exec = nullptr;    // a step of a run: its closing half kick is left to the next replay
+    cudaGraphExec_t whole = nullptr;   // a step by itself (srbe_step of one step)
     cudaEvent_t done = nullptr;
   } slot[2];
   cudaStream_t cap = nullptr;   // capture stream (a legacy default stream cannot be captured)
@@ -411,13 +412,15 @@ struct srbe::HostExt {
   bool graph_dirty = true;
   bool graph_failed = false;
   uint64_t epoch = 0;           // counts calls that may change what a captured step reads
-  int64_t graph_kernels = 0;
+  int64_t graph_kernels = 0, whole_kernels = 0;
+  bool single = false;          // the last srbe_step was of one step
   void drop_graphs() {
     for (auto &sl : slot)
-      if (sl.exec) {
-        cudaGraphExecDestroy(sl.exec);
-        sl.exec = nullptr;
-      }
+      for (cudaGraphExec_t *g : {&sl.exec, &sl.whole})
+        if (*g) {
+          cudaGraphExecDestroy(*g);
+          *g = nullptr;
+        }
     graph_dirty = true;
   }
   // phase tracing: a pool of event pairs, drained into per-phase sums when full or on request
@@ -819,9 +822,11 @@ void check_dev_sampler(srbe_ctx *c) {
   }
 }
 
+enum StepKind { kStepOfRun, kStepWhole, kProviderPass };
+
 // one captured MD step of c.  staged (batch graphs): the mode list is already on the device, and the step
-// is whole.  Otherwise the step leaves its closing half kick to the next replay or to integrate_close.
-void device_step(srbe_ctx *c, int slot, bool staged) {
+// is whole.  A step of a run leaves its closing half kick to the next replay or to integrate_close.
+void device_step(srbe_ctx *c, int slot, bool staged, bool whole) {
   Extra *e = extra(c);
   const int K = c->K;
   SRBE_REQUIRE(c->dm.cap > (size_t)K && c->dc.cap >= (size_t)K && e->slot[slot].dhm, SRBE_ESTATE,
@@ -846,9 +851,14 @@ void device_step(srbe_ctx *c, int slot, bool staged) {
   c->launches++;
   SRBE_CUDA(cudaGetLastError());
   SRBE_CUDA(cudaEventRecord(c->ev_modes, c->side));
-  integrate_close_open(c, c->stepw.p + (1 - slot));
+  if (whole) integrate_open(c);
+  else integrate_close_open(c, c->stepw.p + (1 - slot));
   SRBE_CUDA(cudaStreamWaitEvent(c->stream, c->ev_modes, 0));
   forces_pass(c, false, true);
+  if (whole) {
+    integrate_close(c);
+    return;
+  }
   // the closing half kick is now pending (any non-zero word); on the side stream, beside the force pass
   SRBE_CUDA(cudaMemsetAsync(c->pending.p, 1, sizeof(int), c->side));
   SRBE_CUDA(cudaEventRecord(c->ev_modes, c->side));
@@ -931,7 +941,7 @@ void fill_slot(srbe_ctx *c, int slot) {
   copy_to_slot(c, slot);
 }
 
-// Captures device_step (provider: provider_step) of every context in ctxs into one executable graph
+// Captures device_step (kProviderPass: provider_step) of every context in ctxs into one executable graph
 // per slot.  With width 0
 // all run in order on the capture stream; otherwise context r runs on forks[r % width], forked from
 // and joined back into the capture stream, so that up to width replicas overlap on the GPU.  The
@@ -940,7 +950,7 @@ void fill_slot(srbe_ctx *c, int slot) {
 // Returns false (and leaves nothing captured) when capture is not possible.
 bool capture_graphs(srbe_ctx *const *ctxs, int n, cudaStream_t main, int width, const cudaStream_t *forks,
                     cudaGraphExec_t out[2], int64_t *kernels, DevBuf<StageEntry> *stage_tabs,
-                    bool provider = false) {
+                    StepKind kind = kStepOfRun) {
   std::vector<int64_t> launches0(n);
   for (int r = 0; r < n; ++r) launches0[r] = ctxs[r]->launches;
   std::vector<cudaStream_t> saved(n);
@@ -1003,8 +1013,8 @@ bool capture_graphs(srbe_ctx *const *ctxs, int n, cudaStream_t main, int width, 
           c->stream = main;
         }
         const int64_t l0 = c->launches;
-        if (provider) provider_step(c, slot);
-        else device_step(c, slot, stage_tabs != nullptr);
+        if (kind == kProviderPass) provider_step(c, slot);
+        else device_step(c, slot, stage_tabs != nullptr, kind == kStepWhole);
         kernels[r] = c->launches - l0 + (stage_tabs && r == 0 ? 1 : 0);
         if (width > 0) {
           SRBE_CUDA(cudaEventRecord(join[r], c->stream));
@@ -1793,7 +1803,7 @@ int srbe_forces_host_io(srbe_ctx *c, uint64_t seed, uint64_t step, double *psi_b
       e->drop_io_graphs();
       srbe_ctx *one[1] = {c};
       if (!e->cap) e->cap = make_stream(true);
-      if (capture_graphs(one, 1, e->cap, 0, nullptr, e->io_exec, &e->io_kernels, nullptr, true)) {
+      if (capture_graphs(one, 1, e->cap, 0, nullptr, e->io_exec, &e->io_kernels, nullptr, kProviderPass)) {
         e->io_epoch = e->epoch;
         e->io_K = c->K;
       }
@@ -1837,6 +1847,12 @@ int srbe_step(srbe_ctx *c, int nsteps, uint64_t seed0) {
     report_status(c, false);     // flags that earlier (asynchronous) steps raised
     initial_forces(c, seed0);
     const bool graphs = !c->profiling && c->use_graphs && !e->graph_failed && nsteps > 0;
+    // A step by itself replays a graph with both its half kicks; a run replays graphs that leave the closing one
+    // to the next step.  (A single step as a run of one, with the pending word and a closing launch: 39 against
+    // 34.5 us on the 784-site slab, 72 against 67 on the 11,072-site one, mixed.)  Each is captured when it is first needed,
+    // a single step's after a run only when two of them come in a row.
+    const bool whole = nsteps == 1 && (e->graph_dirty || e->graph_K != c->K || e->slot[0].whole || e->single);
+    e->single = nsteps == 1;
     if (graphs && (e->graph_dirty || e->graph_K != c->K)) {
       // one step the ordinary way sizes every buffer the step touches, then the step is captured
       eager_step(c, seed0);
@@ -1844,15 +1860,18 @@ int srbe_step(srbe_ctx *c, int nsteps, uint64_t seed0) {
       e->drop_graphs();
       reserve(c);
       ensure_slot_buffers(c);
+      e->graph_dirty = false;
+      e->graph_K = c->K;
+    }
+    if (graphs && !(whole ? e->slot[0].whole : e->slot[0].exec)) {
       cudaGraphExec_t ex[2] = {nullptr, nullptr};
       srbe_ctx *one[1] = {c};
       if (!e->cap) e->cap = make_stream(true);
-      if (capture_graphs(one, 1, e->cap, 0, nullptr, ex, &e->graph_kernels, nullptr)) {
-        e->slot[0].exec = ex[0];
-        e->slot[1].exec = ex[1];
-        e->graph_dirty = false;
-        e->graph_K = c->K;
+      if (capture_graphs(one, 1, e->cap, 0, nullptr, ex, whole ? &e->whole_kernels : &e->graph_kernels, nullptr,
+                         whole ? kStepWhole : kStepOfRun)) {
+        for (int k = 0; k < 2; ++k) (whole ? e->slot[k].whole : e->slot[k].exec) = ex[k];
       } else {
+        e->drop_graphs();
         e->graph_failed = true;
       }
     }
@@ -1878,11 +1897,11 @@ int srbe_step(srbe_ctx *c, int nsteps, uint64_t seed0) {
             fill_slot(c, slot);
           }
           coop_before(c);
-          SRBE_CUDA(cudaGraphLaunch(e->slot[slot].exec, c->stream));
-          ++queued;
+          SRBE_CUDA(cudaGraphLaunch(whole ? e->slot[slot].whole : e->slot[slot].exec, c->stream));
+          if (!whole) ++queued;
           coop_after(c);
           SRBE_CUDA(cudaEventRecord(e->slot[slot].done, c->stream));
-          c->launches += e->graph_kernels;
+          c->launches += whole ? e->whole_kernels : e->graph_kernels;
         }
       } catch (...) {
         close();
@@ -1942,9 +1961,9 @@ int srbe_set_graphs(srbe_ctx *c, int on) {
 int srbe_graph_state(srbe_ctx *c, int *captured, int64_t *kernels_per_step) {
   return guarded(c, [&] {
     Extra *e = extra(c);
-    const bool ok = e->slot[0].exec && !e->graph_dirty && !e->graph_failed;
+    const bool run = e->slot[0].exec != nullptr, ok = (run || e->slot[0].whole) && !e->graph_dirty && !e->graph_failed;
     if (captured) *captured = ok ? 1 : (e->graph_failed ? -1 : 0);
-    if (kernels_per_step) *kernels_per_step = ok ? e->graph_kernels : 0;
+    if (kernels_per_step) *kernels_per_step = !ok ? 0 : (run ? e->graph_kernels : e->whole_kernels);
   }, true);
 }
 
