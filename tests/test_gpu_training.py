@@ -89,6 +89,33 @@ def test_prediction_at_tile_edges(ctx):
         last = y
 
 
+@pytest.mark.parametrize("n", [65535, 65536, 66560, 131072, 132098])
+def test_gradients_at_the_chunk_edges(ctx, n):
+    """One chunk of activations less a row, a whole one, one split more, two, and a part of the third."""
+    D, T = rows(n, n)
+    ctx.mlp_init(seed=3)
+    P = ctx.mlp_params()
+    g, loss = ctx.mlp_gradients(D, T)
+    ref_loss, ref = omlp.loss_and_grad(P, D, T)
+    assert rel(g, ref) < 2e-5
+    assert abs(loss - ref_loss) < 2e-5 * ref_loss
+
+
+def test_training_scratch_is_bounded():
+    """Beside the rows themselves a training or gradient call holds at most 172 MB on the device, whatever their
+    number and the minibatch (activations 156 MB, split gradients 7 MB, their sums, the device's 2 MB pages)."""
+    import torch
+    D, T = rows(300000, 1)
+    with srbe.Context((2.0, 2.0, 12.0), 3.5, 0.05, 1.2, 10, 2) as c:
+        c.mlp_init(seed=3)
+        c.mlp_gradients(D[:100], T[:100])
+        c.mlp_predict(D)                       # the rows' own buffer
+        free = torch.cuda.mem_get_info()[0]
+        c.mlp_gradients(D, T)
+        c.mlp_train(D, T, epochs=1, batch=300000, lr=1e-4, seed=2)
+        assert free - torch.cuda.mem_get_info()[0] <= 172 * 10 ** 6
+
+
 def shuffles(n, epochs, seed):
     """Fisher-Yates rows of every epoch, one Philox4x64-10 word per exchange."""
     out, ctr = [], 0
