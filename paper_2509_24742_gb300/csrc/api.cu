@@ -511,17 +511,9 @@ void coop_after(srbe_ctx *c) {
 namespace srbe {
 
 void upload_table(srbe_ctx *c) {
-  std::vector<double2> h(kTab);
-  for (int j = 0; j < kTab; ++j) {
-    const long double a = 2.0L * 3.141592653589793238462643383279502884L * (long double)j / (long double)kTab;
-    h[j] = make_double2((double)cosl(a), (double)sinl(a));
-  }
-  std::vector<longlong2> hi(kTab);
-  fix_table(hi.data());
-  SRBE_CUDA(cudaMemcpyAsync(c->tabi.ensure(kTab), hi.data(), sizeof(longlong2) * kTab, cudaMemcpyHostToDevice,
-                            c->stream));
-  c->tab.ensure(kTab);
-  SRBE_CUDA(cudaMemcpyAsync(c->tab.p, h.data(), sizeof(double2) * kTab, cudaMemcpyHostToDevice, c->stream));
+  const AngleTables &t = angle_tables();
+  SRBE_CUDA(cudaMemcpyAsync(c->tabi.ensure(kTab), t.q, sizeof(t.q), cudaMemcpyHostToDevice, c->stream));
+  SRBE_CUDA(cudaMemcpyAsync(c->tab.ensure(kTab), t.d, sizeof(t.d), cudaMemcpyHostToDevice, c->stream));
   SRBE_CUDA(cudaStreamSynchronize(c->stream));
 }
 

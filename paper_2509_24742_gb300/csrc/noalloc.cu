@@ -111,9 +111,7 @@ int setup_device(DeviceSetup **out) {
   if (!s.ready) {
     if (cudaGetSymbolAddress((void **)&s.scratch, na_scratch) != cudaSuccess) return SRBE_ECUDA;
     if (cudaGetSymbolAddress((void **)&s.table, na_table) != cudaSuccess) return SRBE_ECUDA;
-    longlong2 h[kTab];
-    fix_table(h);
-    if (cudaMemcpyToSymbol(na_table, h, sizeof(h)) != cudaSuccess) return SRBE_ECUDA;
+    if (cudaMemcpyToSymbol(na_table, angle_tables().q, sizeof(angle_tables().q)) != cudaSuccess) return SRBE_ECUDA;
     // A copy from pageable memory may return before its DMA has landed, and streams created
     // non-blocking do not wait for the legacy stream it ran on: wait for it here, so that a first
     // call on any stream reads a complete table.
