@@ -1411,7 +1411,10 @@ int srbe_set_positions(srbe_ctx *c, int64_t n_ion, const double *r, const double
     SRBE_REQUIRE(n_ion < (1ll << 23), SRBE_EINVAL, "at most 8,388,607 ions are supported");
     SRBE_REQUIRE(finite_all(r, 3 * n_ion) && finite_all(q, n_ion), SRBE_EINVAL, "non-finite ion position or charge");
     if (c->have_md && n_ion != c->ni) c->have_md = false;
-    if (n_ion != c->ni) c->nbr.cap = 0;
+    if (n_ion != c->ni) {
+      c->nbr.cap = 0;
+      c->nbr.built = false;
+    }
     Extra *e = extra(c);
     // the same ions with the same charges (an MD engine handing in each step's positions) keep their
     // Verlet lists: the per-step refresh rebuilds them once some ion has moved more than half the
@@ -1452,7 +1455,10 @@ int srbe_set_positions_dev(srbe_ctx *c, int64_t n_ion, const double *r_dev, cons
     SRBE_REQUIRE(n_ion >= 0 && (n_ion == 0 || (r_dev && q_dev)), SRBE_EINVAL, "null positions or charges");
     SRBE_REQUIRE(n_ion < (1ll << 23), SRBE_EINVAL, "at most 8,388,607 ions are supported");
     if (c->have_md && n_ion != c->ni) c->have_md = false;
-    if (n_ion != c->ni) c->nbr.cap = 0;
+    if (n_ion != c->ni) {
+      c->nbr.cap = 0;
+      c->nbr.built = false;
+    }
     c->ni = n_ion;
     neighbor_force_rebuild(c);
     extra(c)->hq.clear();   // charges from device memory: the next host call rebuilds
@@ -2112,6 +2118,10 @@ int srbe_descriptors(srbe_ctx *c, float *D) {
     SRBE_REQUIRE(D, SRBE_EINVAL, "null output");
     SRBE_REQUIRE(c->have_ele && c->have_pos && c->nbr.cap > 0, SRBE_ESTATE,
                  "descriptors need a charge update or force call first");
+    if (!c->nbr.built) {                 // a new skin has changed the lists' capacity since that call
+      reserve(c);
+      neighbor_update(c);
+    }
     c->mlp.D.ensure((size_t)c->ne * mlp_input_width());
     mlp_descriptors(c, c->mlp.D.p);
     SRBE_CUDA(cudaMemcpyAsync(D, c->mlp.D.p, sizeof(float) * c->ne * mlp_input_width(), cudaMemcpyDeviceToHost,
@@ -2317,6 +2327,7 @@ int srbe_set_skin(srbe_ctx *c, double skin) {
     SRBE_REQUIRE(std::isfinite(skin) && skin > 0.0 && skin <= 1.0, SRBE_EINVAL, "skin must be in (0, 1] nm");
     c->nbr.skin = skin;
     c->nbr.cap = 0;                    // list capacity follows the skin (recomputed by reserve)
+    c->nbr.built = false;
     if (c->have_pos) {
       reserve(c);
       neighbor_force_rebuild(c);
@@ -2832,6 +2843,7 @@ int srbe_autotune_skin(srbe_ctx *c, int trial_steps, uint64_t seed, const double
     for (int i = 0; i < n_skins; ++i) {
       c->nbr.skin = skins[i];
       c->nbr.cap = 0;
+      c->nbr.built = false;
       reserve(c);
       neighbor_force_rebuild(c);
       extra(c)->graph_dirty = true;
@@ -2853,6 +2865,7 @@ int srbe_autotune_skin(srbe_ctx *c, int trial_steps, uint64_t seed, const double
     cudaEventDestroy(t1);
     c->nbr.skin = best_skin;
     c->nbr.cap = 0;
+    c->nbr.built = false;
     reserve(c);
     neighbor_force_rebuild(c);
     c->profiling = prof;

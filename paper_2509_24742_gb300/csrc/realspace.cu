@@ -1387,6 +1387,7 @@ void neighbor_update(srbe_ctx *c) {
   SRBE_CUDA(cudaLaunchCooperativeKernel((const void *)k_neighbor_update, dim3(want), dim3(256), args, 0, c->stream));
   coop_after(c);
   c->launches += 2;
+  nb.built = true;
 }
 
 // The period W of the pair coordinates: a power of two with R1 = W / 8 just above rc (and the FP32

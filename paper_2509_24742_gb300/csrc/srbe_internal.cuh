@@ -121,6 +121,7 @@ struct NbrLists {
   DevBuf<int32_t> ii, ie, ei;        // ion-ion [ni][cap], ion-electrode [ni][cap], electrode-ion [ne][cap]
   DevBuf<int32_t> ii_n, ie_n, ei_n;  // entry counts (can exceed cap: the gathers then walk the stencil)
   int cap = 0;
+  bool built = false;                // the lists were built with this cap (a rebuild of them may be due all the same)
   DevBuf<double> xb, yb;             // sorted x, y at the last build (unwrapping reference)
   DevBuf<float4> pfb;                // sorted FP32 positions at the last build
   DevBuf<float4> pm;                 // the same with the molecule id's bits (MD): the list build's candidates
