@@ -1356,6 +1356,12 @@ int srbe_set_electrode(srbe_ctx *c, int64_t n_ele, const double *R, const int8_t
       (side[j] ? nr : nl)++;
     }
     SRBE_REQUIRE(nl > 0 && nr > 0, SRBE_EINVAL, "both electrodes need at least one site");
+    // until all of it is set there is no electrode, and the lists of an earlier one (its sites, its cells) are no
+    // lists of this
+    c->have_ele = false;
+    c->nbr.cap = 0;
+    c->nbr.built = false;
+    neighbor_force_rebuild(c);
     c->ne = n_ele;
     c->hR.assign(R, R + 3 * n_ele);
     c->hside.assign(side, side + n_ele);
@@ -1401,6 +1407,9 @@ int srbe_set_electrode(srbe_ctx *c, int64_t n_ele, const double *R, const int8_t
     lattice_setup(c, x, y, z);
     build_A_and_inverse(c);
     c->have_ele = true;
+    // an iterative solve chosen for an earlier electrode goes on with this one's matrix and sizes
+    if (c->pcg.on && c->dense) pcg_prepare(c);
+    else c->pcg.on = false;
     extra(c)->forces_valid = false;
   });
 }

@@ -24,3 +24,33 @@ def test_descriptors_after_a_new_skin(precision):
             c.set_skin(skin)
             E = c.descriptors()
             assert np.abs(E - D).max() <= 2e-5 * np.abs(D).max()
+
+
+@pytest.mark.parametrize("precision,solver", [(srbe.FP64, srbe.DIRECT), (srbe.MIXED, srbe.DIRECT), (srbe.FP64, srbe.PCG),
+                                              (srbe.MIXED, srbe.PCG)])
+def test_another_electrode_on_the_same_context(precision, solver):
+    """srbe_set_electrode again, with more and with fewer sites, over the same ions: the next pass is a fresh
+    context's, bit for bit (lists built anew by both, an iterative solve from a zero start)."""
+    a = wl.make_slab("first", (2.26, 2.02, 12.0), 9, 8, 39, 3, alpha=3.5, eta_inv=19.79, rc=1.2, P=40, M=2, seed=3,
+                     placement="lattice")
+    c = srbe.from_slab(a, precision=precision, alpha_A=1.7)
+    for nx, ny, gone in ((9, 8, 0), (10, 9, 0), (6, 7, 1), (10, 9, 3)):
+        s = wl.make_slab("next", a.box, nx, ny, 39, 3, alpha=3.5, eta_inv=19.79, rc=1.2, P=40, M=2, seed=3,
+                         placement="lattice")
+        s.r, s.q = a.r, a.q
+        s.R, s.side = s.R[gone:], s.side[gone:]
+        out = []
+        for ctx in (c, srbe.from_slab(s, precision=precision, alpha_A=1.7)):
+            if ctx is c:
+                ctx.set_electrode(s.R, s.side)
+            if solver == srbe.PCG and (ctx is not c or nx == 9):
+                ctx.set_solver(srbe.PCG, tol=1e-10, maxit=4000, warm=srbe.WARM_ZERO)
+            ctx.sample_k(5, 1)
+            out.append(ctx.forces()[:2])
+            if ctx is not c:
+                ctx.close()
+        assert all(np.array_equal(x, y) for x, y in zip(*out))
+    with pytest.raises(srbe.SrbeError):
+        c.set_electrode(s.R, np.zeros_like(s.side))          # one side empty: refused, the electrode stays
+    assert np.array_equal(c.forces()[0], out[0][0])
+    c.close()
