@@ -307,8 +307,9 @@ int srbe_mlp_train(srbe_ctx *ctx, const float *D, const float *target, int64_t n
  * charges of the last pass, ||A Q - dpsi d - b - psi_bar e|| / ||dpsi d + b|| (A Q = dpsi d + b +
  * psi_bar e follows from Eqs. 9-10), with A in FP64 whatever the precision of the solve.
  * srbe_set_skin / srbe_get_skin: Verlet-list skin (nm, default 0.1); lists hold pairs within rc +
- * skin and are rebuilt on the device once an ion has moved more than skin / 2.  Results do not
- * depend on the skin beyond summation order.
+ * skin and are rebuilt on the device once an ion has moved more than skin / 2 (for a skin larger than
+ * the one at srbe_set_electrode: than half of what its cells' stencil covers beyond rc, if that is less).
+ * Results do not depend on the skin beyond summation order.
  * srbe_autotune_skin: times trial_steps MD steps (after two untimed ones) for each candidate skin,
  * restores positions, velocities, forces, charges and the step counter after each trial, keeps the
  * fastest skin and writes the per-candidate ms per step to ms_per_step (n_skins entries, or NULL). */

@@ -1365,7 +1365,14 @@ void neighbor_update(srbe_ctx *c) {
   a.z0f = (float)cl.g.z0;
   const float reach = (float)(c->rc + nb.skin) + (c->precision == SRBE_MIXED ? 0.f : kPrecheckMargin);
   a.cut2 = reach * reach;
-  a.half_skin2 = (float)(0.25 * nb.skin * nb.skin);
+  // the stencil was chosen for the skin at srbe_set_electrode: where a larger one reaches beyond it, the lists are
+  // complete only up to the stencil, and the rebuild comes after half of what that leaves
+  double skin = nb.skin;
+  for (int d = 0; d < 3; ++d) {
+    const double cover = cl.g.span[d] * cl.g.cs[d] - c->rc;
+    if (cover < skin - 1e-9) skin = std::max(cover, 0.0);
+  }
+  a.half_skin2 = (float)(0.25 * skin * skin);
   a.flag = nb.flag.p;
   static int blocks_per_sm = 0, nsm = 0;
   if (!blocks_per_sm) {

@@ -54,3 +54,40 @@ def test_another_electrode_on_the_same_context(precision, solver):
         c.set_electrode(s.R, np.zeros_like(s.side))          # one side empty: refused, the electrode stays
     assert np.array_equal(c.forces()[0], out[0][0])
     c.close()
+
+
+def test_skin_beyond_the_stencil():
+    """Cells are chosen for the default skin (0.1 nm): in a box of 4 nm they are 2/3 nm wide and two of them cover
+    1.333 nm, so lists for rc + 0.3 nm lack some pairs.  Ions that start 1.34 to 1.49 nm apart and come within rc by
+    moving less than half the skin each are seen all the same: a fresh context's forces."""
+    rng = np.random.default_rng(4)
+    s = wl.make_slab("skin", (4.0, 4.0, 12.0), 8, 8, 60, 1, alpha=2.0, eta_inv=19.79, rc=1.2, P=30, M=2, seed=3,
+                     placement="lattice")
+    s.r, s.q = s.r[:40].copy(), s.q[:40]
+    s.r[:, 2] = 2.2 + 1.9 * (np.arange(40) // 20)
+    for k in range(20):
+        for h in (0, 1):
+            s.r[2 * k + h, :2] = [(0.66 + (k % 5) * 0.79 + h * 0.0) % 4.0, (k % 4) + 0.01]
+        d = rng.normal(size=2)
+        s.r[2 * k + 1, :2] += (1.34 + 0.15 * rng.random()) * d / np.linalg.norm(d)
+    far = s.r.copy()
+    near = s.r.copy()
+    for k in range(20):
+        d = far[2 * k + 1] - far[2 * k]
+        u = 0.145 * d / np.linalg.norm(d)
+        near[2 * k] += u
+        near[2 * k + 1] -= u
+    with srbe.from_slab(s, alpha_A=1.7) as c:
+        c.set_skin(0.3)
+        c.sample_k(5, 1)
+        c.forces()
+        c.set_positions(near, s.q)             # the same ions: the lists are kept while they hold
+        F, Q, _ = c.forces()
+    t = copy.copy(s)
+    t.r = near
+    with srbe.from_slab(t, alpha_A=1.7) as c:
+        c.sample_k(5, 1)
+        F2, Q2, _ = c.forces()
+    # the same pairs in another order: sums of a few hundred FP64 terms
+    assert np.abs(F - F2).max() <= 1e-11 * np.abs(F2).max()
+    assert np.abs(Q - Q2).max() <= 1e-11 * np.abs(Q2).max()
