@@ -308,9 +308,9 @@ __global__ void k_sfac_reduce(SfFinish f) {
 // over more particles, while shorter ones give more blocks to hide latency with.  occ is a context
 // setting (default 8) that srbe_autotune_tiles / srbe_batch_autotune_tiles choose by timing.
 // The FP64 form spends ten times as long on a particle, so while there are fewer than two blocks per SM its
-// chunks shrink to 64 or 32 particles: 3,072 sites, 204 modes (168 blocks, 16 SMs with two of them): 24.9 ->
-// 18.0 us; 400 particles, 102 modes: 23.2 -> 11.8 us.  Four blocks per SM as the line is slower (8,000
-// particles 29 -> 34 us: each block ends with a reduction and a fence).
+// chunks shrink to 64 or 32 particles: 3,072 sites, 204 modes (168 blocks, 16 SMs with two of them): 22.0 ->
+// 18.3 us; 400 particles, 102 modes: 20.6 -> 11.9 us (this rule alone, ncu).  Four blocks per SM as the line is
+// slower (8,000 particles 29 -> 34 us: each block ends with a reduction and a fence).
 int64_t sfac_chunks(int64_t n, int K, int occ, bool fp64, int64_t *chunk) {
   static int nsm = 0;
   if (!nsm) {

@@ -137,9 +137,9 @@ k_descriptors(int64_t ne, const double *__restrict__ ex, const double *__restric
 // 40 KB operand buffer holds X and then, since X is dead once Z1 is complete, each half of H1 in turn
 // (64 columns: K steps 0-3, then 4-7 of the second layer), so that the weights (104 KB) and both
 // groups fit the shared memory.  The next tile's rows are loaded into registers while the first layer
-// runs.  The weights come already split and blocked from k_mlp_split (once per set of parameters).
+// runs.  The weights come already split and blocked from k_mlp_split.
 // 98,304 rows: 33 us; 66 us with one tile in flight per SM, the weights split by every CTA and IEEE divisions in
-// the SiLU and the standardisation.  3,072 rows: 26.5 -> 13 us.  The quotients are corrected ones (sfu.cuh): with
+// the SiLU and the standardisation.  3,072 rows: 26.5 -> 14 us.  The quotients are corrected ones (sfu.cuh): with
 // plain products by the reciprocal (30 us) the error against 64 bits was 1.0012 +- 0.0003 of the divisions' over
 // 80 networks of 4,000 rows, with the correction 1.0001 +- 0.0001 (6.84e-6, which is the BF16 split's).
 // ------------------------------------------------------------------------------------------------

@@ -1053,7 +1053,10 @@ __global__ void __launch_bounds__(256, 1) k_pcg_mixed(PcgArgs a) {
     }
     if (it >= a.maxit) break;
     // the inner residual's target: 1e-4 of the outer one, but no less than a quarter of the tolerance, and
-    // that directly where it is at most 1e-5 away (a further correction would mostly overshoot it)
+    // that directly where it is at most 1e-5 away.  Corrections of 1e-4 each end anywhere below the tolerance: over
+    // six electrodes of 987 to 3,072 sites, cold and learned starts, tolerance 1e-8, at residuals of 1e-12 to 8.5e-9
+    // (charges up to 2.5e-8 off the direct solve's) after 45 to 118 iterations; so at 1.1e-9 to 2.5e-9 (up to 9.6e-9
+    // off) after 49 to 93.
     const double goal = 0.0625 * a.tol2 * vv;
     const float stop = (float)(goal >= 1e-10 * rr ? goal : 1e-8 * rr);
     if (a.srows) {
