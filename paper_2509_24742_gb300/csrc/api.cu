@@ -2364,7 +2364,7 @@ struct Snapshot {
 
 void snapshot_io(srbe_ctx *c, Snapshot &sn, bool save) {
   const size_t n = (size_t)c->ni, ne = (size_t)c->ne;
-  if (save) sn.pcg = c->pcg.y.p != nullptr;
+  if (save) sn.pcg = c->pcg.on;     // (else its iterate may be of an earlier electrode's size, and nothing reads it)
   const bool pcg = sn.pcg;
   SRBE_REQUIRE(!pcg || c->pcg.y.p, SRBE_ESTATE, "PCG state vanished under a snapshot");
   double *b = save ? sn.buf.ensure(9 * n + ne + (pcg ? ne : 0) + 1) : sn.buf.p;

@@ -91,3 +91,21 @@ def test_skin_beyond_the_stencil():
     # the same pairs in another order: sums of a few hundred FP64 terms
     assert np.abs(F - F2).max() <= 1e-11 * np.abs(F2).max()
     assert np.abs(Q - Q2).max() <= 1e-11 * np.abs(Q2).max()
+
+
+def test_autotune_after_another_electrode():
+    """The tuners save and restore the state of trial steps.  The iterate of an iterative solve that is no longer
+    selected is no part of it: it has the size of the electrode it was used with."""
+    a, b = (wl.make_slab("tune", (2.26, 2.02, 12.0), nx, ny, 39, 3, alpha=3.5, eta_inv=19.79, rc=1.2, P=40, M=2, seed=3,
+                         with_md=True, placement="lattice") for nx, ny in ((6, 5), (10, 9)))
+    with srbe.from_slab(a, precision=srbe.MIXED, alpha_A=1.7, md=True) as c:
+        c.minimize(10)
+        c.set_solver(srbe.PCG, tol=1e-8, maxit=2000, warm=srbe.WARM_PREVIOUS)
+        c.step(2, 3)
+        c.set_solver(srbe.DIRECT)
+        c.set_electrode(b.R, b.side)
+        r, v = c.get_positions(velocities=True)
+        c.autotune_skin(2, 3, skins=(0.05, 0.1))
+        c.autotune_tiles(2, 3, occ=(4, 8))
+        r2, v2 = c.get_positions(velocities=True)
+    assert np.array_equal(r, r2) and np.array_equal(v, v2)
